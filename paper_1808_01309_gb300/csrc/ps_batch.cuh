@@ -54,6 +54,8 @@ template <typename T, int N>
 __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v), MinB<T, N>::xpass)
     k_batch_xpass(const __grid_constant__ BatchArgs B, const int M, const int rpc) {
   using V = typename cplx<T>::type;
+  using FV = typename fft_of<V>::val;
+  using W = typename fft_of<V>::tw;
   constexpr int E = EPass<T, N, 3>::v, G = N / E;
   constexpr int NF = 6;
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -69,7 +71,7 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v), MinB
   const long long total = ng * M;
   V* stage = reinterpret_cast<V*>(smraw);
   V* exbuf = stage + NF * rpc * kxp;
-  LinesExchange<V, 1> ex{exbuf + rl * XLINES * N, N, 0, 0};
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLINES * N, N, 0, 0};
   if (G >= 32) {
     ex.bar_id = 1 + rl;
     ex.nthr = G;
@@ -79,17 +81,17 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v), MinB
   // every member has the same twiddles (same nx): those of member 0
   constexpr bool TR = XTwReg<T, N>::v;
   constexpr bool TT = !TR && XTwTable<T, N>::v;
-  using TwAcc = typename std::conditional<TR, RegTw<V, N, E>,
-                typename std::conditional<TT, ThreadTw<V, N, E>, GlobalTw<V>>::type>::type;
+  using TwAcc = typename std::conditional<TR, RegTw<W, N, E>,
+                typename std::conditional<TT, ThreadTw<W, N, E>, GlobalTw<W>>::type>::type;
   TwAcc tw;
   if constexpr (TR) {
-    tw.load(static_cast<const V*>(B.args[0].tw_x), j0);
+    tw.load(static_cast<const W*>(B.args[0].tw_x), j0);
   } else if constexpr (TT) {
-    V* twt = exbuf + rpc * XLINES * N;
-    if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const V*>(B.args[0].tw_x), j0);
+    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLINES * N);
+    if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const W*>(B.args[0].tw_x), j0);
     tw = TwAcc{twt, j0};
   } else {
-    tw = TwAcc{static_cast<const V*>(B.args[0].tw_x)};
+    tw = TwAcc{static_cast<const W*>(B.args[0].tw_x)};
   }
   if (tid == 0) {
     mbar_init(&bar[0], 1);

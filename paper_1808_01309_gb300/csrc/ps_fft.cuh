@@ -18,6 +18,8 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <type_traits>
+#include "ps_fix.cuh"
 
 namespace ps {
 
@@ -70,11 +72,35 @@ __device__ __forceinline__ float2 cscale(float2 a, float s) {
 }
 #endif
 
+// rot16 below on fixed-point values.
+template <int S16, int DIR>
+__device__ __forceinline__ fx2 rot16_fix(fx2 v) {
+  if constexpr (S16 == 0) {
+    return v;
+  } else if constexpr (S16 == 4) {
+    return DIR > 0 ? cmul_i(v) : cmul_mi(v);
+  } else if constexpr (S16 == 2 || S16 == 6) {
+    const long long p = fx_mul(v.x + v.y, FX_HH, FX_HL), m = fx_mul(v.x - v.y, FX_HH, FX_HL);
+    if constexpr (S16 == 2) return DIR > 0 ? mk<fx2>(m, p) : mk<fx2>(p, -m);
+    else return DIR > 0 ? mk<fx2>(-p, m) : mk<fx2>(-m, -p);
+  } else {
+    constexpr bool big = S16 == 1 || S16 == 7;  // |cos| = cos(pi/8)
+    constexpr int sg = S16 > 4 ? -1 : 1;
+    fxw w;
+    w.xh = sg * (big ? FX_C1H : FX_S1H);
+    w.xl = sg * (big ? FX_C1L : FX_S1L);
+    w.yh = DIR * (big ? FX_S1H : FX_C1H);
+    w.yl = DIR * (big ? FX_S1L : FX_C1L);
+    return cmul(v, w);
+  }
+}
+
 // Multiply by exp(DIR * 2 pi i * s/16) for a compile-time s in [0, 8).
 // cos(pi/8), sin(pi/8) and sqrt(1/2) are the exact mathematical constants,
 // rounded by the compiler to the working precision.
 template <int S16, int DIR, typename V>
 __device__ __forceinline__ V rot16(V v) {
+  if constexpr (std::is_same<V, fx2>::value) return rot16_fix<S16, DIR>(v);
   using T = decltype(V::x);
   constexpr double C1 = 0.92387953251128675612818318939678828682;  // cos(pi/8)
   constexpr double S1 = 0.38268343236508977172845998403039886676;  // sin(pi/8)
@@ -149,8 +175,14 @@ __device__ __forceinline__ void dft3(V& a, V& b, V& c) {
   using T = decltype(V::x);
   constexpr double S3 = 0.86602540378443864676372317075293618347;  // sqrt(3)/2
   const V t1 = cadd(b, c);
-  const V t2 = csub(a, cscale(t1, T(0.5)));
-  const V d = cscale(csub(b, c), T(DIR * S3));
+  V t2, d = csub(b, c);
+  if constexpr (std::is_same<V, fx2>::value) {
+    t2 = mk<V>(a.x - ((t1.x + 1) >> 1), a.y - ((t1.y + 1) >> 1));
+    d = mk<V>(fx_mul(d.x, DIR * FX_S3H, DIR * FX_S3L), fx_mul(d.y, DIR * FX_S3H, DIR * FX_S3L));
+  } else {
+    t2 = csub(a, cscale(t1, T(0.5)));
+    d = cscale(d, T(DIR * S3));
+  }
   a = cadd(a, t1);
   b = cadd(t2, cmul_i(d));
   c = csub(t2, cmul_i(d));
@@ -169,8 +201,19 @@ __device__ __forceinline__ void dft(V (&x)[R]) {
     V e0 = x[0], e1 = x[2], e2 = x[4], o0 = x[1], o1 = x[3], o2 = x[5];
     dft3<DIR>(e0, e1, e2);
     dft3<DIR>(o0, o1, o2);
-    o1 = cmul(o1, mk<V>(T(0.5), T(DIR * S3)));   // w6
-    o2 = cmul(o2, mk<V>(T(-0.5), T(DIR * S3)));  // w6^2
+    if constexpr (std::is_same<V, fx2>::value) {
+      fxw w;
+      w.xh = FX_5H;
+      w.xl = 0;
+      w.yh = DIR * FX_S3H;
+      w.yl = DIR * FX_S3L;
+      o1 = cmul(o1, w);  // w6
+      w.xh = -FX_5H;
+      o2 = cmul(o2, w);  // w6^2
+    } else {
+      o1 = cmul(o1, mk<V>(T(0.5), T(DIR * S3)));   // w6
+      o2 = cmul(o2, mk<V>(T(-0.5), T(DIR * S3)));  // w6^2
+    }
     x[0] = cadd(e0, o0);
     x[3] = csub(e0, o0);
     x[1] = cadd(e1, o1);
@@ -214,12 +257,22 @@ template <typename T, int N> struct EOf {
 // the non-coherent path) or a copy in shared memory.  at<NS, R>(r, b, idx)
 // returns the twiddle of input r of the thread's butterfly b in the stage with
 // previous radix product NS, which is tw[idx].
+template <typename V> __device__ __forceinline__ V ldg_tw(const V* p) { return __ldg(p); }
+__device__ __forceinline__ fxw ldg_tw(const fxw* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  fxw w;
+  w.xh = v.x;
+  w.xl = v.y;
+  w.yh = v.z;
+  w.yl = v.w;
+  return w;
+}
 template <typename V>
 struct GlobalTw {
   const V* __restrict__ p;
-  __device__ __forceinline__ V operator[](int i) const { return __ldg(p + i); }
+  __device__ __forceinline__ V operator[](int i) const { return ldg_tw(p + i); }
   template <int NS, int R>
-  __device__ __forceinline__ V at(int, int, int idx) const { return __ldg(p + idx); }
+  __device__ __forceinline__ V at(int, int, int idx) const { return ldg_tw(p + idx); }
 };
 template <typename V>
 struct SharedTw {
@@ -273,7 +326,7 @@ struct RegTw {
     for (int b = 0; b < NB; ++b) {
       const int k = (j0 + b * (N / E)) % NS;
 #pragma unroll
-      for (int r = 1; r < R; ++r) w[TwSlots<N, E>::base(NS) + b * (R - 1) + (r - 1)] = __ldg(tw + r * k * (N / (NS * R)));
+      for (int r = 1; r < R; ++r) w[TwSlots<N, E>::base(NS) + b * (R - 1) + (r - 1)] = ldg_tw(tw + r * k * (N / (NS * R)));
     }
   }
   __device__ __forceinline__ void load(const V* __restrict__ tw, int j0) {
@@ -328,7 +381,7 @@ __device__ __forceinline__ void stage(V (&a)[E], int j0, const TW& tw, X& ex) {
     if constexpr (NS > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const V w = tw.template at<NS, R>(r, b, r * k * (N / (NS * R)));
+        const auto w = tw.template at<NS, R>(r, b, r * k * (N / (NS * R)));
         x[r] = cmul(x[r], DIR > 0 ? cconj(w) : w);
       }
     }
@@ -371,13 +424,6 @@ __device__ __forceinline__ void line_fft_tw(V (&a)[E], int j0, const TW& tw, X& 
   }
 }
 
-// Full length-N line transform with twiddles read from global memory.
-template <int N, int E, int DIR, typename V, class X>
-__device__ __forceinline__ void line_fft(V (&a)[E], int j0, const V* __restrict__ twp, X& ex) {
-  const GlobalTw<V> tw{twp};
-  line_fft_tw<N, E, DIR>(a, j0, tw, ex);
-}
-
 // Shared-memory exchange for lines laid out as columns: element n of line l
 // at buf[row(n) * LP + l].  With NBUF = 2 two buffers are used alternately so
 // that one barrier per exchange suffices (a buffer is rewritten only after the
@@ -385,8 +431,10 @@ __device__ __forceinline__ void line_fft(V (&a)[E], int j0, const V* __restrict_
 // its reads); with NBUF = 1 a second barrier after the reads frees the single
 // buffer.  row(n) flips the lowest bit when bit SW of n is set: the first
 // exchange writes rows R1 apart, and this keeps them on alternate bank halves.
-template <typename V, int SW, int NBUF = 2>
+// TX: lines side by side (lp; 0 where only FP32 lines are transformed).
+template <typename V, int SW, int NBUF = 2, int TX = 0>
 struct ColumnExchange {
+  static constexpr int cols = TX;
   V* buf;
   int bufsz;
   int lp;
@@ -476,6 +524,71 @@ struct LinesExchange {
   }
 };
 
+// Bound of sum |re| + |im| over the line from its threads' parts u, for lines
+// laid out as columns: TX lines side by side, thread = line + TX (j0 + G b).
+// Every thread of the CTA calls it; the lines of a CTA exchange at least once
+// between two calls, so the shared words of a call are read before the next
+// call writes them.
+template <int TX, int G>
+__device__ __forceinline__ int fx_column_bound(int u) {
+  if constexpr (TX * G <= 32) {
+    return fx_lane_sum<TX, TX * G>(u);
+  } else {
+    constexpr int W = TX * G / 32;  // warps of a line
+    __shared__ int part[32 * TX];
+    u = fx_lane_sum<TX, 32>(u);
+    const int w = threadIdx.x >> 5, l = threadIdx.x % TX;
+    if ((threadIdx.x & 31) < TX) part[w * TX + l] = u;
+    __syncthreads();
+    const int w0 = w / W * W;
+    u = part[w0 * TX + l];
+#pragma unroll
+    for (int i = 1; i < W; ++i) u = fx_add_bound(u, part[(w0 + i) * TX + l]);
+    return u;
+  }
+}
+// The same for the NL lines of a row spread over G consecutive threads.
+template <int G, int NL, class X>
+__device__ __forceinline__ void fx_row_bounds(int (&u)[NL], X& ex) {
+#pragma unroll
+  for (int l = 0; l < NL; ++l) u[l] = fx_lane_sum<1, (G < 32 ? G : 32)>(u[l]);
+  if constexpr (G > 32) {
+    constexpr int W = G / 32;
+    __shared__ int part[32 * 3];
+    static_assert(NL <= 3, "lines of a row transformed together");
+    const int w = threadIdx.x >> 5, w0 = w / W * W;
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+      for (int l = 0; l < NL; ++l) part[w * 3 + l] = u[l];
+    ex.sync();
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      u[l] = part[w0 * 3 + l];
+#pragma unroll
+      for (int i = 1; i < W; ++i) u[l] = fx_add_bound(u[l], part[(w0 + i) * 3 + l]);
+    }
+  }
+}
+
+// Full length-N transform of a column line with twiddles read from global
+// memory (FP64: in block fixed point, ps_fix.cuh).
+template <int N, int E, int DIR, typename V, class X>
+__device__ __forceinline__ void line_fft(V (&a)[E], int j0, const void* twp, X& ex) {
+  using W = typename fft_of<V>::tw;
+  const GlobalTw<W> tw{static_cast<const W*>(twp)};
+  if constexpr (std::is_same<V, double2>::value) {
+    static_assert(X::cols > 0, "columns of the tile");
+    const FxScale sc = fx_scale(fx_column_bound<X::cols, N / E>(fx_partial(a)));
+    fx2 b[E];
+    fx_load(b, a, sc);
+    line_fft_tw<N, E, DIR>(b, j0, tw, ex);
+#pragma unroll
+    for (int m = 0; m < E; ++m) a[m] = fx_value(b[m], sc);
+  } else {
+    line_fft_tw<N, E, DIR>(a, j0, tw, ex);
+  }
+}
+
 // One Stockham stage (as in stage()) applied to NL independent lines held by
 // the same threads: the butterflies of all lines are issued together (the
 // stage twiddles are shared), then one exchange moves all lines.
@@ -486,11 +599,12 @@ __device__ __forceinline__ void stage_rows(V (&a)[NL][E], int j0, const TW& tw, 
   for (int b = 0; b < NB; ++b) {
     const int j = j0 + b * (N / E);
     const int k = j % NS;
-    V w[R];
+    using W = typename std::decay<decltype(tw.template at<NS, R>(0, 0, 0))>::type;
+    W w[R];
     if constexpr (NS > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const V t = tw.template at<NS, R>(r, b, r * k * (N / (NS * R)));
+        const W t = tw.template at<NS, R>(r, b, r * k * (N / (NS * R)));
         w[r] = DIR > 0 ? cconj(t) : t;
       }
     }
@@ -542,6 +656,51 @@ __device__ __forceinline__ void line_fft_rows(V (&a)[NL][E], int j0, const TW& t
     stage_rows<N, E, S::R2, S::R0 * S::R1, DIR, false>(a, j0, tw, ex);
     stage_rows<N, E, S::R3, S::R0 * S::R1 * S::R2, DIR, true>(a, j0, tw, ex);
   }
+}
+
+// The lines before and after line_fft_rows: FP32 values as they are; FP64
+// values in block fixed point, with the scale of each line.
+template <int N, int E, int NL, class X>
+__device__ __forceinline__ void rows_load(float2 (&b)[NL][E], const float2 (&a)[NL][E], FxScale (&)[NL], X&) {
+#pragma unroll
+  for (int l = 0; l < NL; ++l)
+#pragma unroll
+    for (int m = 0; m < E; ++m) b[l][m] = a[l][m];
+}
+template <int N, int E, int NL, class X>
+__device__ __forceinline__ void rows_load(fx2 (&b)[NL][E], const double2 (&a)[NL][E], FxScale (&sc)[NL], X& ex) {
+  int u[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) u[l] = fx_partial(a[l]);
+  fx_row_bounds<N / E>(u, ex);
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    sc[l] = fx_scale(u[l]);
+    fx_load(b[l], a[l], sc[l]);
+  }
+}
+// One value of a transformed line, halved if HALF.
+template <bool HALF = false>
+__device__ __forceinline__ float2 line_value(float2 v, FxScale) {
+  if constexpr (HALF) return cscale(v, 0.5f);
+  return v;
+}
+template <bool HALF = false>
+__device__ __forceinline__ double2 line_value(fx2 v, FxScale sc) {
+  if constexpr (HALF) sc.s += 1;
+  return fx_value(v, sc);
+}
+// Transform of NL lines in place.
+template <int N, int E, int DIR, int NL, typename V, class TW, class X>
+__device__ __forceinline__ void rows_fft(V (&a)[NL][E], int j0, const TW& tw, X& ex) {
+  typename fft_of<V>::val b[NL][E];
+  FxScale sc[NL];
+  rows_load<N>(b, a, sc, ex);
+  line_fft_rows<N, E, DIR>(b, j0, tw, ex);
+#pragma unroll
+  for (int l = 0; l < NL; ++l)
+#pragma unroll
+    for (int m = 0; m < E; ++m) a[l][m] = line_value(b[l][m], sc[l]);
 }
 
 }  // namespace ps

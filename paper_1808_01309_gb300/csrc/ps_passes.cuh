@@ -262,8 +262,8 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   const int kx = tl.x() * TX + line;  // local column
   const int kxg = g.kx0 + kx;              // its global kx
   const int q = iy <= g.Ky ? iy : iy - g.cy;
-  ColumnExchange<V, ilog2<Sched<N, E>::R0>::v, 1> ex{xbuf + bb * N * TX, 0, TX, line, 0};
-  const V* tw = static_cast<const V*>(a.tw_z);
+  using FV = typename fft_of<V>::val;
+  ColumnExchange<FV, ilog2<Sched<N, E>::R0>::v, 1, TX> ex{reinterpret_cast<FV*>(xbuf) + bb * N * TX, 0, TX, line, 0};
   V* out = static_cast<V*>(a.a6);
   const T skx = T(kxg) * pick<T>(g.sx, g.sxf), sky = T(q) * pick<T>(g.sy, g.syf), sz = pick<T>(g.sz, g.szf);
   const long long fstride = (long long)g.nz * g.cy * g.kxp;
@@ -362,7 +362,7 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
       x[m] = v;
     }
     if (a.e_part && f < 3) esum += (double)ssq;
-    line_fft<N, E, +1>(x, j0, tw, ex);
+    line_fft<N, E, +1>(x, j0, a.tw_z, ex);
     if (bvalid) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
@@ -394,7 +394,8 @@ __device__ __forceinline__ void yinv_tile(const PassArgs& a, const TL& tl) {
   using SH = ColShape<T, N, 1, VAR>;
   constexpr int E = SH::E, G = SH::G, TX = SH::TX, NB = SH::NB;
   extern __shared__ __align__(128) unsigned char smraw[];
-  V* sm = reinterpret_cast<V*>(smraw);
+  using FV = typename fft_of<V>::val;
+  FV* sm = reinterpret_cast<FV*>(smraw);
   const Geo& g = a.g;
   const int tid = threadIdx.x;
   const int line = tid % TX, rest = tid / TX, j0 = rest % G, bb = rest / G;
@@ -402,7 +403,7 @@ __device__ __forceinline__ void yinv_tile(const PassArgs& a, const TL& tl) {
   const bool bvalid = iz < g.nz;
   const int kx = tl.x() * TX + line;
   const int f = tl.z();
-  ColumnExchange<V, ilog2<Sched<N, E>::R0>::v, ColBuf<T, N>::v> ex{sm + bb * N * TX, NB * N * TX, TX, line, 0};
+  ColumnExchange<FV, ilog2<Sched<N, E>::R0>::v, ColBuf<T, N>::v, TX> ex{sm + bb * N * TX, NB * N * TX, TX, line, 0};
   const V* in = static_cast<const V*>(a.a6) + ((long long)f * g.nz + (bvalid ? iz : 0)) * g.cy * g.kxp + kx;
   V* out = static_cast<V*>(a.b6) + ((long long)f * g.nz + (bvalid ? iz : 0)) * g.ny * g.kxp + kx;
   V x[E];
@@ -414,7 +415,7 @@ __device__ __forceinline__ void yinv_tile(const PassArgs& a, const TL& tl) {
     if (bvalid && q <= g.Ky && q >= -g.Ky) v = ldv<COH>(in + (long long)rowof(q, g.cy) * g.kxp);
     x[m] = v;
   }
-  line_fft<N, E, +1>(x, j0, static_cast<const V*>(a.tw_y), ex);
+  line_fft<N, E, +1>(x, j0, a.tw_y, ex);
   if (bvalid) {
 #pragma unroll
     for (int m = 0; m < E; ++m) out[(long long)(j0 + m * (N / E)) * g.kxp] = x[m];
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(ColShape<T, N, 1, VAR>::NTH, MinB<T, N>::ypass
 template <typename T, int N, int NG, int NSC, bool COH, class TW, class AfterGather, int XE = EPass<T, N, 3>::v>
 __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row, const bool rvalid, const int j0,
                                           const typename cplx<T>::type* st, const long long fst, const TW& tw,
-                                          LinesExchange<typename cplx<T>::type, 1>& ex, T& umax2,
+                                          LinesExchange<typename fft_of<typename cplx<T>::type>::val, 1>& ex, T& umax2,
                                           AfterGather&& gathered) {
   using V = typename cplx<T>::type;
   constexpr int E = XE;
@@ -499,7 +500,7 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
   }
   gathered();
   if constexpr (HD) {
-    line_fft_rows<N, E, +1>(U, j0, tw, ex);
+    rows_fft<N, E, +1>(U, j0, tw, ex);
   } else if constexpr (NSC == 1) {
     V L[3][E], S[2][E];
 #pragma unroll
@@ -510,8 +511,8 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
     for (int c = 0; c < 2; ++c)
 #pragma unroll
       for (int m = 0; m < E; ++m) S[c][m] = U[3 + c][m];
-    line_fft_rows<N, E, +1>(L, j0, tw, ex);
-    line_fft_rows<N, E, +1>(S, j0, tw, ex);
+    rows_fft<N, E, +1>(L, j0, tw, ex);
+    rows_fft<N, E, +1>(S, j0, tw, ex);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -528,7 +529,7 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
       for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int m = 0; m < E; ++m) L[c][m] = U[3 * h + c][m];
-      line_fft_rows<N, E, +1>(L, j0, tw, ex);
+      rows_fft<N, E, +1>(L, j0, tw, ex);
 #pragma unroll
       for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -564,7 +565,11 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
     }
   }
   if (!a.xdiag) {  // uniform across the grid
-    line_fft_rows<N, E, -1>(F, j0, tw, ex);
+    using FV = typename fft_of<V>::val;
+    FV H[NFW][E];
+    FxScale sc[NFW];
+    rows_load<N>(H, F, sc, ex);
+    line_fft_rows<N, E, -1>(H, j0, tw, ex);
     const long long rrow = rvalid ? row : 0;
     const int kend = kxp < N / 2 + 1 ? kxp : N / 2 + 1;
     // split each packed transform F = DFT(a) + i DFT(b) of two real fields
@@ -574,7 +579,7 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
 #pragma unroll
     for (int w = 0; w < NSP; ++w)
 #pragma unroll
-      for (int m = 0; m < E; ++m) ex.template put<0, 0>(w, j0 + m * (N / E), F[w][m]);
+      for (int m = 0; m < E; ++m) ex.template put<0, 0>(w, j0 + m * (N / E), H[w][m]);
     ex.sync();
 #pragma unroll
     for (int w = 0; w < NFW; ++w) {
@@ -587,13 +592,13 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
         if (rvalid && k < kend) {
           V va = czero<V>(), vb = czero<V>();
           if (k <= g.Kx) {
-            const V Fk = F[w][m];
+            const FV Fk = H[w][m];
             if (split) {
-              const V Fm = cconj(ex.template get<0, 0>(w, k == 0 ? 0 : N - k));
-              va = cscale(cadd(Fk, Fm), T(0.5));
-              vb = cscale(cmul_mi(csub(Fk, Fm)), T(0.5));
+              const FV Fm = cconj(ex.template get<0, 0>(w, k == 0 ? 0 : N - k));
+              va = line_value<true>(cadd(Fk, Fm), sc[w]);
+              vb = line_value<true>(cmul_mi(csub(Fk, Fm)), sc[w]);
             } else {
-              va = Fk;
+              va = line_value(Fk, sc[w]);
             }
           }
           ca[k] = va;
@@ -609,6 +614,8 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v),
                                   NG == 1 && NSC == 0 ? MinB<T, N>::xpass : 1)
     k_xpass(const PassArgs a, const int rpc) {
   using V = typename cplx<T>::type;
+  using FV = typename fft_of<V>::val;
+  using W = typename fft_of<V>::tw;
   constexpr int E = EPass<T, N, 3>::v, G = N / E;
   constexpr int NF = 6 * NG + 3 * NSC;  // input fields: u, omega (, B, j) (, grad theta)
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -624,7 +631,7 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v),
   V* stage = reinterpret_cast<V*>(smraw);
   V* exbuf = stage + NF * rpc * kxp;
   // exchange region of this row: XLINES lines of N slots, single buffer
-  LinesExchange<V, 1> ex{exbuf + rl * XLINES * N, N, 0, 0};
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLINES * N, N, 0, 0};
   // rows are independent between the group barriers: sync only the row's threads
   if (G >= 32) {
     ex.bar_id = 1 + rl;
@@ -636,17 +643,17 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v),
   // memory (thread j0 of every row reads its own column), else global memory
   constexpr bool TR = XTwReg<T, N>::v;
   constexpr bool TT = !TR && XTwTable<T, N>::v;
-  using TwAcc = typename std::conditional<TR, RegTw<V, N, E>,
-                typename std::conditional<TT, ThreadTw<V, N, E>, GlobalTw<V>>::type>::type;
+  using TwAcc = typename std::conditional<TR, RegTw<W, N, E>,
+                typename std::conditional<TT, ThreadTw<W, N, E>, GlobalTw<W>>::type>::type;
   TwAcc tw;
   if constexpr (TR) {
-    tw.load(static_cast<const V*>(a.tw_x), j0);
+    tw.load(static_cast<const W*>(a.tw_x), j0);
   } else if constexpr (TT) {
-    V* twt = exbuf + rpc * XLINES * N;
-    if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const V*>(a.tw_x), j0);
+    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLINES * N);
+    if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const W*>(a.tw_x), j0);
     tw = TwAcc{twt, j0};
   } else {
-    tw = TwAcc{static_cast<const V*>(a.tw_x)};
+    tw = TwAcc{static_cast<const W*>(a.tw_x)};
   }
   const V* B = static_cast<const V*>(a.b6);
   if (tid == 0) {
@@ -720,7 +727,8 @@ __device__ __forceinline__ void yfwd_tile(const PassArgs& a, const TL& tl) {
   using SH = ColShape<T, N, 1, VAR>;
   constexpr int E = SH::E, G = SH::G, TX = SH::TX, NB = SH::NB;
   extern __shared__ __align__(128) unsigned char smraw[];
-  V* sm = reinterpret_cast<V*>(smraw);
+  using FV = typename fft_of<V>::val;
+  FV* sm = reinterpret_cast<FV*>(smraw);
   const Geo& g = a.g;
   const int tid = threadIdx.x;
   const int line = tid % TX, rest = tid / TX, j0 = rest % G, bb = rest / G;
@@ -728,13 +736,13 @@ __device__ __forceinline__ void yfwd_tile(const PassArgs& a, const TL& tl) {
   const bool bvalid = iz < g.nz;
   const int kx = tl.x() * TX + line;
   const int f = tl.z();
-  ColumnExchange<V, ilog2<Sched<N, E>::R0>::v, ColBuf<T, N>::v> ex{sm + bb * N * TX, NB * N * TX, TX, line, 0};
+  ColumnExchange<FV, ilog2<Sched<N, E>::R0>::v, ColBuf<T, N>::v, TX> ex{sm + bb * N * TX, NB * N * TX, TX, line, 0};
   const V* in = static_cast<const V*>(a.a6) + ((long long)f * g.nz + (bvalid ? iz : 0)) * g.ny * g.kxp + kx;
   V* out = static_cast<V*>(a.b6) + ((long long)f * g.nz + (bvalid ? iz : 0)) * g.cy * g.kxp + kx;
   V x[E];
 #pragma unroll
   for (int m = 0; m < E; ++m) x[m] = bvalid ? ldv<COH>(in + (long long)(j0 + m * (N / E)) * g.kxp) : czero<V>();
-  line_fft<N, E, -1>(x, j0, static_cast<const V*>(a.tw_y), ex);
+  line_fft<N, E, -1>(x, j0, a.tw_y, ex);
   if (bvalid) {
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -761,7 +769,8 @@ __device__ __forceinline__ void zfwd_tile(const PassArgs& a, const TL& tl) {
   using SH = ColShape<T, N, 2, VAR>;
   constexpr int E = SH::E, G = SH::G, TX = SH::TX, NB = SH::NB;
   extern __shared__ __align__(128) unsigned char smraw[];
-  V* sm = reinterpret_cast<V*>(smraw);
+  using FV = typename fft_of<V>::val;
+  FV* sm = reinterpret_cast<FV*>(smraw);
   const Geo& g = a.g;
   const int tid = threadIdx.x;
   const int line = tid % TX, rest = tid / TX, j0 = rest % G, bb = rest / G;
@@ -770,14 +779,14 @@ __device__ __forceinline__ void zfwd_tile(const PassArgs& a, const TL& tl) {
   const int kx = tl.x() * TX + line;
   const int q = iy <= g.Ky ? iy : iy - g.cy;
   const int f = tl.z();
-  ColumnExchange<V, ilog2<Sched<N, E>::R0>::v, ColBuf<T, N>::v> ex{sm + bb * N * TX, NB * N * TX, TX, line, 0};
+  ColumnExchange<FV, ilog2<Sched<N, E>::R0>::v, ColBuf<T, N>::v, TX> ex{sm + bb * N * TX, NB * N * TX, TX, line, 0};
   const long long cs_in = (long long)g.nz * g.cy * g.kxp;
   const V* in = static_cast<const V*>(a.b6) + f * cs_in + (long long)(bvalid ? iy : 0) * g.kxp + kx;
   V x[E];
 #pragma unroll
   for (int m = 0; m < E; ++m)
     x[m] = bvalid ? ldv<COH>(in + (long long)(j0 + m * (N / E)) * g.cy * g.kxp) : czero<V>();
-  line_fft<N, E, -1>(x, j0, static_cast<const V*>(a.tw_z), ex);
+  line_fft<N, E, -1>(x, j0, a.tw_z, ex);
   if (bvalid) {
     const T inv = pick<T>(a.inv_n3, a.inv_n3f);
     V* out = static_cast<V*>(a.a6) + (long long)f * g.cz * g.cy * g.kxp + (long long)iy * g.kxp + kx;

@@ -95,16 +95,18 @@ __device__ __forceinline__ void ens_xpass_tile(const PassArgs& a, const int tile
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ double red[32];
   const int tid = threadIdx.x, j0 = tid % G, rl = tid / G;
-  LinesExchange<V, 1> ex{reinterpret_cast<V*>(smraw) + rl * XLINES * N, N, 0, 0};
+  using FV = typename fft_of<V>::val;
+  using W = typename fft_of<V>::tw;
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(smraw) + rl * XLINES * N, N, 0, 0};
   ex.bar_id = -1;
-  const GlobalTw<V> tw{static_cast<const V*>(a.tw_x)};
+  const GlobalTw<W> tw{static_cast<const W*>(a.tw_x)};
   const long long rows = (long long)a.g.nz * a.g.ny;
   const long long row = (long long)tile * RPC + rl;
   const bool rvalid = row < rows;
   const V* B = static_cast<const V*>(a.b6) + (rvalid ? row : 0) * a.g.kxp;
   T umax2 = 0;
   auto none = [] {};
-  xpass_row<T, N, 1, 0, true, GlobalTw<V>, decltype(none)&, E>(a, row, rvalid, j0, B, rows * a.g.kxp, tw, ex, umax2,
+  xpass_row<T, N, 1, 0, true, GlobalTw<W>, decltype(none)&, E>(a, row, rvalid, j0, B, rows * a.g.kxp, tw, ex, umax2,
                                                                 none);
   if (a.umax2) {
     const double t = block_max((double)umax2, red);

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "ps.h"
+#include "ps_fix.cuh"
 #include "ps_kernels.h"
 
 using namespace ps;
@@ -464,14 +465,18 @@ void fill_twiddles(std::vector<V>& out, int n) {
     out.push_back(v);
   }
 }
+// The FP64 passes' twiddles in block fixed point.
+void fill_twiddles(std::vector<ps::fxw>& out, int n) {
+  for (int m = 0; m < n; ++m) out.push_back(ps::fx_twiddle(m, n));
+}
 
 template <typename V>
 ps_status upload_twiddles(ps_plan* p) {
-  std::vector<V> h;
+  std::vector<typename ps::fft_of<V>::tw> h;
   fill_twiddles(h, p->g.nx);
   fill_twiddles(h, p->g.ny);
   fill_twiddles(h, p->g.nz);
-  PS_CU(cudaMemcpy(p->tw, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice), "twiddle upload");
+  PS_CU(cudaMemcpy(p->tw, h.data(), h.size() * sizeof(h[0]), cudaMemcpyHostToDevice), "twiddle upload");
   return PS_OK;
 }
 
@@ -1289,11 +1294,11 @@ ps_status ps_slab_create(const ps_config* cfg, int kx_lo, int kx_hi, int z_lo, i
     fill_twiddles(h, g.nz);
     e = cudaMemcpy(s->tw, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice);
   } else {
-    std::vector<double2> h;
+    std::vector<ps::fxw> h;
     fill_twiddles(h, g.nx);
     fill_twiddles(h, g.ny);
     fill_twiddles(h, g.nz);
-    e = cudaMemcpy(s->tw, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice);
+    e = cudaMemcpy(s->tw, h.data(), h.size() * sizeof(ps::fxw), cudaMemcpyHostToDevice);
   }
   if (e != cudaSuccess) return bail(cuda_fail(e, "slab twiddle upload"));
   if (cfg->forcing) {

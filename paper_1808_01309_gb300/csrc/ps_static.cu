@@ -41,7 +41,14 @@ cudaError_t scratch_address(void** out) {
   return cudaSuccess;
 }
 
-// exp(-2 pi i m/n), m < n, for the three axes, from the FP64 sincospi.
+// exp(-2 pi i m/n), m < n, for the three axes: FP32 passes from the FP64
+// sincospi, FP64 passes in block fixed point.
+__device__ void twiddle(float2& w, int m, int n) {
+  double s, c;
+  sincospi(2.0 * m / n, &s, &c);
+  w = make_float2((float)c, (float)(-s));
+}
+__device__ void twiddle(fxw& w, int m, int n) { w = fx_twiddle(m, n); }
 template <typename V>
 __global__ void k_twiddles(V* tw, int nx, int ny, int nz) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -58,12 +65,7 @@ __global__ void k_twiddles(V* tw, int nx, int ny, int nz) {
     m = i - nx - ny;
     n = nz;
   }
-  double s, c;
-  sincospi(2.0 * m / n, &s, &c);
-  V v;
-  v.x = (decltype(v.x))c;
-  v.y = (decltype(v.x))(-s);
-  tw[i] = v;
+  twiddle(tw[i], m, n);
 }
 
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
@@ -129,7 +131,8 @@ ps_status run(const ps_config* c, cudaStream_t s, const void* uhat, void* out) {
   a.g = g;
   a.a6 = p;
   a.b6 = p + a_b;
-  V* tw = reinterpret_cast<V*>(p + a_b + b_b);
+  using W = typename fft_of<V>::tw;
+  W* tw = reinterpret_cast<W*>(p + a_b + b_b);
   a.tw_x = tw;
   a.tw_y = tw + g.nx;
   a.tw_z = tw + g.nx + g.ny;
@@ -156,7 +159,7 @@ ps_status run(const ps_config* c, cudaStream_t s, const void* uhat, void* out) {
   // this call's output into NaN (the update kernel reads the word)
   if ((e = cudaMemsetAsync(a.err, 0, sizeof(int), s)) != cudaSuccess) return cuda_bad(e, "error word");
   const int ntw = g.nx + g.ny + g.nz;
-  k_twiddles<V><<<(ntw + 255) / 256, 256, 0, s>>>(tw, g.nx, g.ny, g.nz);
+  k_twiddles<W><<<(ntw + 255) / 256, 256, 0, s>>>(tw, g.nx, g.ny, g.nz);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_bad(e, "twiddles");
   if (c->forcing) {
     // the whole retained cube as the forcing box: no extent query, no sync
