@@ -27,10 +27,11 @@ __global__ void k_tw(V* tw, int n) {
   tw[m] = make_float2((float)c, (float)(-s));
 }
 
-// In-place C2C transform along an axis of length N: element n of line
-// (b, col) at (b / nb2) s1 + (b % nb2) s2 + n es + col, col < ncols.
+// C2C transform along an axis of length N: element n of line (b, col) at
+// (b / nb2) s1 + (b % nb2) s2 + n es + col, col < ncols, of src and dst (which
+// may be the same array: a CTA holds its lines before it stores them).
 template <int N, int DIR>
-__global__ void k_c2c(V* data, const V* __restrict__ tw, int ncols, int nb2, long long s1, long long s2,
+__global__ void k_c2c(const V* src, V* dst, const V* __restrict__ tw, int ncols, int nb2, long long s1, long long s2,
                       long long es, int nbatch) {
   constexpr int E = EOf<float, N>::v, G = N / E;
   constexpr int NBG = 256 / (TXG * G) > 0 ? 256 / (TXG * G) : 1;
@@ -42,10 +43,12 @@ __global__ void k_c2c(V* data, const V* __restrict__ tw, int ncols, int nb2, lon
   const int col = blockIdx.x * TXG + line;
   const bool ok = b < nbatch && col < ncols;
   ColumnExchange<V, ilog2<Sched<N, E>::R0>::v> ex{sm + bb * N * TXG, NBG * N * TXG, TXG, line, 0};
-  V* base = data + (ok ? (long long)(b / nb2) * s1 + (long long)(b % nb2) * s2 + col : 0);
+  const long long off = ok ? (long long)(b / nb2) * s1 + (long long)(b % nb2) * s2 + col : 0;
+  const V* from = src + off;
+  V* base = dst + off;
   V x[E];
 #pragma unroll
-  for (int m = 0; m < E; ++m) x[m] = ok ? base[(long long)(j0 + m * (N / E)) * es] : czero<V>();
+  for (int m = 0; m < E; ++m) x[m] = ok ? from[(long long)(j0 + m * (N / E)) * es] : czero<V>();
   line_fft<N, E, DIR>(x, j0, tw, ex);
   if (ok) {
 #pragma unroll
@@ -132,7 +135,7 @@ __global__ void k_r2c(const float* __restrict__ phys, V* __restrict__ spec, cons
 }
 
 template <int N, int DIR>
-cudaError_t c2c_n(V* data, const V* tw, int ncols, int nb2, long long s1, long long s2, long long es, int nbatch,
+cudaError_t c2c_n(const V* src, V* dst, const V* tw, int ncols, int nb2, long long s1, long long s2, long long es, int nbatch,
                   cudaStream_t s) {
   constexpr int E = EOf<float, N>::v, G = N / E;
   constexpr int NBG = 256 / (TXG * G) > 0 ? 256 / (TXG * G) : 1;
@@ -142,7 +145,7 @@ cudaError_t c2c_n(V* data, const V* tw, int ncols, int nb2, long long s1, long l
     if (e != cudaSuccess) return e;
   }
   dim3 grid((ncols + TXG - 1) / TXG, (nbatch + NBG - 1) / NBG);
-  k_c2c<N, DIR><<<grid, TXG * G * NBG, smem, s>>>(data, tw, ncols, nb2, s1, s2, es, nbatch);
+  k_c2c<N, DIR><<<grid, TXG * G * NBG, smem, s>>>(src, dst, tw, ncols, nb2, s1, s2, es, nbatch);
   return cudaGetLastError();
 }
 
@@ -188,14 +191,14 @@ cudaError_t r2c_n(const float* phys, V* spec, const V* tw, int F, long long rows
     default: return cudaErrorInvalidValue;     \
   }
 
-cudaError_t c2c(int n, int dir, V* d, const V* tw, int ncols, int nb2, long long s1, long long s2, long long es,
+cudaError_t c2c(int n, int dir, const V* f, V* d, const V* tw, int ncols, int nb2, long long s1, long long s2, long long es,
                 int nbatch, cudaStream_t s) {
   if (dir > 0) {
-#define CALL(N) c2c_n<N, +1>(d, tw, ncols, nb2, s1, s2, es, nbatch, s)
+#define CALL(N) c2c_n<N, +1>(f, d, tw, ncols, nb2, s1, s2, es, nbatch, s)
     LES_DISPATCH(n, CALL)
 #undef CALL
   } else {
-#define CALL(N) c2c_n<N, -1>(d, tw, ncols, nb2, s1, s2, es, nbatch, s)
+#define CALL(N) c2c_n<N, -1>(f, d, tw, ncols, nb2, s1, s2, es, nbatch, s)
     LES_DISPATCH(n, CALL)
 #undef CALL
   }
@@ -212,13 +215,14 @@ cudaError_t r2c(int n, const float* phys, V* spec, const V* tw, int F, long long
 #undef CALL
 }
 
-// Spectral [F][nz][ny][nh] (overwritten by the z and y passes) -> physical
-// [F][nz][ny][nx], unnormalised backward sum.
-cudaError_t spec2phys(const Geo& g, int F, V* spec, float* phys, const V* twx, const V* twy, const V* twz,
+// Spectral src [F][nz][ny][nh] -> physical [F][nz][ny][nx], unnormalised
+// backward sum; spec (src itself or a second array) holds the z and y passes'
+// results.
+cudaError_t spec2phys(const Geo& g, int F, const V* src, V* spec, float* phys, const V* twx, const V* twy, const V* twz,
                       cudaStream_t s) {
   const long long plane = (long long)g.ny * g.nh, fs = (long long)g.nz * plane;
-  cudaError_t e = c2c(g.nz, +1, spec, twz, g.nh, g.ny, fs, g.nh, plane, F * g.ny, s);
-  if (e == cudaSuccess) e = c2c(g.ny, +1, spec, twy, g.nh, g.nz, fs, plane, g.nh, F * g.nz, s);
+  cudaError_t e = c2c(g.nz, +1, src, spec, twz, g.nh, g.ny, fs, g.nh, plane, F * g.ny, s);
+  if (e == cudaSuccess) e = c2c(g.ny, +1, spec, spec, twy, g.nh, g.nz, fs, plane, g.nh, F * g.nz, s);
   if (e == cudaSuccess) e = c2r(g.nx, spec, phys, twx, F, (long long)g.nz * g.ny, s);
   return e;
 }
@@ -229,8 +233,8 @@ cudaError_t phys2spec(const Geo& g, int F, const float* phys, V* spec, const V* 
   const long long plane = (long long)g.ny * g.nh, fs = (long long)g.nz * plane;
   const float scale = (float)(1.0 / ((double)g.nx * g.ny * g.nz));
   cudaError_t e = r2c(g.nx, phys, spec, twx, F, (long long)g.nz * g.ny, scale, s);
-  if (e == cudaSuccess) e = c2c(g.ny, -1, spec, twy, g.nh, g.nz, fs, plane, g.nh, F * g.nz, s);
-  if (e == cudaSuccess) e = c2c(g.nz, -1, spec, twz, g.nh, g.ny, fs, g.nh, plane, F * g.ny, s);
+  if (e == cudaSuccess) e = c2c(g.ny, -1, spec, spec, twy, g.nh, g.nz, fs, plane, g.nh, F * g.nz, s);
+  if (e == cudaSuccess) e = c2c(g.nz, -1, spec, spec, twz, g.nh, g.ny, fs, g.nh, plane, F * g.ny, s);
   return e;
 }
 
@@ -515,7 +519,7 @@ cudaError_t les_closure_term(const Geo& g, Spec in, const void* twx, const void*
   const V *tx = static_cast<const V*>(twx), *ty = static_cast<const V*>(twy), *tz = static_cast<const V*>(twz);
   k_grad<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, in, s.spec);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.phys, tx, ty, tz, st);
+  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.spec, s.phys, tx, ty, tz, st);
   if (e == cudaSuccess) {
     k_features<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(s.phys, s.X, nullptr, P, s.norm);
     e = cudaGetLastError();
@@ -548,7 +552,7 @@ cudaError_t les_closure_grad(const Geo& g, Spec in, Spec f, const void* twx, con
   // divergence (compact), as in les_closure_term
   k_grad<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, in, s.spec);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.phys, tx, ty, tz, st);
+  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.spec, s.phys, tx, ty, tz, st);
   if (e == cudaSuccess) {
     k_features<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(s.phys, s.X, s.Arows, P, s.norm);
     e = cudaGetLastError();
@@ -597,7 +601,7 @@ cudaError_t les_closure_grad(const Geo& g, Spec in, Spec f, const void* twx, con
     k_grad<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, r, s.spec);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.phys, tx, ty, tz, st);
+  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.spec, s.phys, tx, ty, tz, st);
   // adjoint through the tensor basis, then the network
   if (e == cudaSuccess) {
     k_dg<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(s.Arows, s.phys, s.norm, (float)(2.0 / (double)P), s.Y, P);
@@ -617,18 +621,144 @@ __global__ void k_rows6(const float* __restrict__ f, float* __restrict__ T, long
   for (int m = 0; m < 6; ++m) T[p * 6 + m] = f[m * P + p];
 }
 
-// u_i u_j (order 11, 22, 33, 12, 13, 23) of 3 planar fields u into 6 fields uu;
-// may run in place with u = uu + 3P (each point reads its three values first).
-__global__ void k_products(const float* u, float* uu, long long P) {
-  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  const float a = u[p], b = u[P + p], c = u[2 * P + p];
-  uu[p] = a * a;
-  uu[P + p] = b * b;
-  uu[2 * P + p] = c * c;
-  uu[3 * P + p] = a * b;
-  uu[4 * P + p] = a * c;
-  uu[5 * P + p] = b * c;
+// u_i u_j (order 11, 22, 33, 12, 13, 23) along x: the half-spectra rows of three
+// fields (N/2+1 modes) -> the modes p < cw of the six products' rows, times
+// scale.  Neither the velocity nor the products ever reach memory in physical
+// space: two packed backward lines (u_1 + i u_2, u_3), three packed forward ones.
+template <int N>
+__global__ void __launch_bounds__(128, 3) k_xprod(const V* __restrict__ u, V* __restrict__ uu, const V* __restrict__ tw,
+                                               long long rows, int cw, float scale) {
+  constexpr int E = EOf<float, N>::v, G = N / E, NH = N / 2 + 1;
+  constexpr int RPC = 128 / G;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  const int j0 = threadIdx.x % G, rl = threadIdx.x / G;
+  const long long row = (long long)blockIdx.x * RPC + rl;
+  const bool ok = row < rows;
+  LinesExchange<V, 1> ex{reinterpret_cast<V*>(smraw) + rl * 3 * N, N, 0, 0};
+  if (G >= 32) {
+    ex.bar_id = 1 + rl;
+    ex.nthr = G;
+  } else {
+    ex.bar_id = -1;
+  }
+  const GlobalTw<V> twa{tw};
+  const V* pu = u + (ok ? row : 0) * NH;
+  V U[2][E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int n = j0 + m * (N / E);
+    const bool hi = n > N / 2;
+    const int p = hi ? N - n : n;
+    V A = czero<V>(), B = czero<V>(), D = czero<V>();
+    if (ok) {
+      A = __ldg(pu + p);
+      B = __ldg(pu + rows * NH + p);
+      D = __ldg(pu + 2 * rows * NH + p);
+    }
+    if (hi) {
+      A = cconj(A);
+      B = cconj(B);
+      D = cconj(D);
+    }
+    U[0][m] = mk<V>(A.x - B.y, A.y + B.x);
+    U[1][m] = D;
+  }
+  line_fft_rows<N, E, +1>(U, j0, twa, ex);
+  V F[3][E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const float a = U[0][m].x, b = U[0][m].y, c = U[1][m].x;
+    F[0][m] = mk<V>(a * a, b * b);
+    F[1][m] = mk<V>(c * c, a * b);
+    F[2][m] = mk<V>(a * c, b * c);
+  }
+  line_fft_rows<N, E, -1>(F, j0, twa, ex);
+#pragma unroll
+  for (int w = 0; w < 3; ++w)
+#pragma unroll
+    for (int m = 0; m < E; ++m) ex.template put<0, 0>(w, j0 + m * (N / E), F[w][m]);
+  ex.sync();
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int p = j0 + m * (N / E);
+    if (ok && p < cw) {
+#pragma unroll
+      for (int w = 0; w < 3; ++w) {
+        const V Fm = cconj(ex.template get<0, 0>(w, p == 0 ? 0 : N - p));
+        uu[(2 * w * rows + row) * cw + p] = cscale(cadd(F[w][m], Fm), 0.5f * scale);
+        uu[((2 * w + 1) * rows + row) * cw + p] = cscale(cmul_mi(csub(F[w][m], Fm)), 0.5f * scale);
+      }
+    }
+  }
+}
+
+// Forward transform along y (Z = false) or z of the six products' modes
+// p < cw, of which only |q|, |r| <= K = cw - 1 are kept (c2 = 2K + 1 each).
+//   y: src [6][n][n][cw] -> dst [6][n][c2][cw]
+//   z: src [6][n][c2][cw] -> the modes of a full-layout spectrum on an nl^3
+//      grid, dst [6][nl][nl][nl/2+1]; sub: subtracted from what is there
+template <int N, bool Z>
+__global__ void k_fwd_keep(const V* __restrict__ src, V* __restrict__ dst, const V* __restrict__ tw, int cw, int nl,
+                           int sub) {
+  constexpr int E = EOf<float, N>::v, G = N / E;
+  constexpr int NBG = 256 / (TXG * G) > 0 ? 256 / (TXG * G) : 1;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  V* sm = reinterpret_cast<V*>(smraw);
+  const int tid = threadIdx.x;
+  const int line = tid % TXG, rest = tid / TXG, j0 = rest % G, bb = rest / G;
+  const int K = cw - 1, c2 = 2 * K + 1;
+  const int nb2 = Z ? c2 : N;  // lines per field and column: retained ky (z pass), or planes
+  const int b = blockIdx.y * NBG + bb, f = b / nb2, i = b % nb2;
+  const int col = blockIdx.x * TXG + line;
+  const bool ok = b < 6 * nb2 && col < cw;
+  ColumnExchange<V, ilog2<Sched<N, E>::R0>::v> ex{sm + bb * N * TXG, NBG * N * TXG, TXG, line, 0};
+  const long long es = Z ? (long long)c2 * cw : cw;
+  const V* from = src + (ok ? (Z ? (long long)f * N * c2 * cw + (long long)i * cw : (long long)b * N * cw) + col : 0);
+  V x[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) x[m] = ok ? __ldg(from + (long long)(j0 + m * (N / E)) * es) : czero<V>();
+  line_fft<N, E, -1>(x, j0, tw, ex);
+  if (!ok) return;
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int r = sidx(j0 + m * (N / E), N);
+    if (r > K || r < -K) continue;
+    if constexpr (Z) {
+      const int q = i <= K ? i : i - c2;
+      V* o = dst + (((long long)f * nl + rowof(r, nl)) * nl + rowof(q, nl)) * (nl / 2 + 1) + col;
+      *o = sub ? csub(*o, x[m]) : x[m];
+    } else {
+      dst[((long long)b * c2 + rowof(r, c2)) * cw + col] = x[m];
+    }
+  }
+}
+
+template <int N>
+cudaError_t products_n(const V* u, V* xb, V* yb, V* out, const V* tw, int kc, int nl, int sub, cudaStream_t s) {
+  constexpr int E = EOf<float, N>::v, G = N / E, RPC = 128 / G;
+  constexpr int NBG = 256 / (TXG * G) > 0 ? 256 / (TXG * G) : 1;
+  const long long rows = (long long)N * N;
+  const int cw = kc + 1, c2 = 2 * kc + 1;
+  const size_t sx = 3ull * RPC * N * sizeof(V), sc = 2ull * NBG * N * TXG * sizeof(V);
+  cudaError_t e = prep(k_xprod<N>, sx);
+  if (e == cudaSuccess) e = prep(k_fwd_keep<N, false>, sc);
+  if (e == cudaSuccess) e = prep(k_fwd_keep<N, true>, sc);
+  if (e != cudaSuccess) return e;
+  k_xprod<N><<<(unsigned)((rows + RPC - 1) / RPC), RPC * G, sx, s>>>(u, xb, tw, rows, cw,
+                                                                     (float)(1.0 / ((double)N * N * N)));
+  const unsigned tx = (cw + TXG - 1) / TXG;
+  k_fwd_keep<N, false><<<dim3(tx, (6 * N + NBG - 1) / NBG), TXG * G * NBG, sc, s>>>(xb, yb, tw, cw, nl, 0);
+  k_fwd_keep<N, true><<<dim3(tx, (6 * c2 + NBG - 1) / NBG), TXG * G * NBG, sc, s>>>(yb, out, tw, cw, nl, sub);
+  return cudaGetLastError();
+}
+// The modes |p|, |q|, |r| <= kc of F[u_i u_j] on an n^3 grid, from the three
+// fields u after their z and y passes, into the full-layout spectra out of an
+// nl^3 grid (zero elsewhere already); xb and yb: scratch of 6 n^2 (kc + 1) and
+// 6 n (2 kc + 1)(kc + 1) modes.
+cudaError_t products(int n, const V* u, V* xb, V* yb, V* out, const V* tw, int kc, int nl, int sub, cudaStream_t s) {
+#define CALL(N) products_n<N>(u, xb, yb, out, tw, kc, nl, sub, s)
+  LES_DISPATCH(n, CALL)
+#undef CALL
 }
 
 // Copy the modes |p|,|q|,|r| <= kc of F full-layout fields on grid gs into
@@ -647,12 +777,6 @@ __global__ void k_truncate(const V* __restrict__ src, const Geo gs, V* __restric
     v = src[f * ts + ((long long)rowof(r, gs.nz) * gs.ny + rowof(q, gs.ny)) * gs.nh + p];
   }
   dst[i] = v;
-}
-
-// a <- a - b on F fields of one grid (full layout).
-__global__ void k_sub(V* __restrict__ a, const V* __restrict__ b, long long n) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) a[i] = csub(a[i], b[i]);
 }
 
 Geo cube_geo(int n) {
@@ -692,112 +816,96 @@ extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int
       if (!(norm12[i] > 0) || !std::isfinite(norm12[i])) return bad("ps_les_training_sample: std must be positive");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const Geo gd = cube_geo(n_dns), gl = cube_geo(n_les);
-  const long long Md = (long long)gd.nz * gd.ny * gd.nh, Pd = (long long)n_dns * n_dns * n_dns;
+  const long long Md = (long long)gd.nz * gd.ny * gd.nh;
   const long long Ml = (long long)gl.nz * gl.ny * gl.nh, Pl = (long long)n_les * n_les * n_les;
-  std::vector<void*> bufs;
-  auto alloc = [&](size_t bytes) -> void* {
-    void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
-    bufs.push_back(p);
-    return p;
+  // one allocation, cut into the transforms' buffers
+  const long long cw = kc + 1, c2 = 2 * kc + 1;
+  size_t need = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = need;
+    need += (bytes + 255) / 256 * 256;
+    return at;
   };
-  V* twd = static_cast<V*>(alloc(sizeof(V) * n_dns));
-  V* twl = static_cast<V*>(alloc(sizeof(V) * n_les));
-  V* sd = static_cast<V*>(alloc(sizeof(V) * 6 * Md));              // DNS spectra (6 fields)
-  float* pd = static_cast<float*>(alloc(sizeof(float) * 6 * Pd));  // DNS physical (6 fields)
-  V* sl = static_cast<V*>(alloc(sizeof(V) * 6 * Ml));              // LES spectra (6 fields)
-  V* sg = static_cast<V*>(alloc(sizeof(V) * 9 * Ml));              // LES spectra (9 fields)
-  float* pl = static_cast<float*>(alloc(sizeof(float) * 9 * Pl));  // LES physical (9 fields)
-  float* nrm = static_cast<float*>(alloc(sizeof(float) * 12));
+  const size_t o_twd = take(sizeof(V) * n_dns), o_twl = take(sizeof(V) * n_les);
+  const size_t o_sd = take(sizeof(V) * 3 * Md);                   // DNS velocity after its z and y passes
+  const size_t o_xb = take(sizeof(V) * 6 * n_dns * n_dns * cw);   // products after the x pass (either grid)
+  const size_t o_yb = take(sizeof(V) * 6 * n_dns * c2 * cw);      // and after the y pass
+  const size_t o_ub = take(sizeof(V) * 3 * Ml);                   // ubar on the LES grid
+  const size_t o_sl = take(sizeof(V) * 6 * Ml);                   // F[u_i u_j] - F[ubar_i ubar_j] on the LES grid
+  const size_t o_sg = take(sizeof(V) * 9 * Ml);                   // transform scratch (9 fields)
+  const size_t o_pl = take(sizeof(float) * 9 * Pl);               // LES physical (9 fields)
+  const size_t o_nrm = take(sizeof(float) * 12);
+  char* base = nullptr;
   ps_status st = PS_OK;
-  if (!twd || !twl || !sd || !pd || !sl || !sg || !pl || !nrm) {
+  if (cudaMalloc(&base, need) != cudaSuccess) {
+    (void)cudaGetLastError();
     set_last_error("ps_les_training_sample: device allocation failed");
-    st = PS_ERR_OOM;
+    return PS_ERR_OOM;
   }
-  cudaError_t e = cudaSuccess;
-  const unsigned bd = blocks(Pd), bl = blocks(Pl);
-  const size_t ubytes = sizeof(V) * 3 * Md;
-  if (st == PS_OK) {
-    float h[12];
-    for (int i = 0; i < 5; ++i) {
-      h[i] = norm12 ? (float)norm12[i] : 0.f;
-      h[5 + i] = norm12 ? (float)(1.0 / norm12[5 + i]) : 1.f;
-    }
-    h[10] = h[11] = 1.f;
-    e = cudaMemcpyAsync(nrm, h, sizeof(h), cudaMemcpyHostToDevice, s);
-    k_tw<<<(n_dns + 255) / 256, 256, 0, s>>>(twd, n_dns);
-    k_tw<<<(n_les + 255) / 256, 256, 0, s>>>(twl, n_les);
-    // 1. F[u_i u_j] on the LES grid: DNS velocity (fields 3..5 of pd), the
-    //    products in place, forward, truncate
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sd, uhat_dns, ubytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = spec2phys(gd, 3, sd, pd + 3 * Pd, twd, twd, twd, s);
-    if (e == cudaSuccess) {
-      k_products<<<bd, 256, 0, s>>>(pd + 3 * Pd, pd, Pd);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = phys2spec(gd, 6, pd, sd, twd, twd, twd, s);
-    if (e == cudaSuccess) {
-      k_truncate<<<blocks(6 * Ml), 256, 0, s>>>(sd, gd, sl, gl, kc, 6);
-      e = cudaGetLastError();
-    }
-    // 2. F[ubar_i ubar_j]: ubar on the LES grid (3 < 2/3 of the grid, so its
-    //    products do not alias below kc), products, forward, truncate
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sd, uhat_dns, ubytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) {
-      k_truncate<<<blocks(3 * Ml), 256, 0, s>>>(sd, gd, sg, gl, kc, 3);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = spec2phys(gl, 3, sg, pl + 3 * Pl, twl, twl, twl, s);
-    if (e == cudaSuccess) {
-      k_products<<<bl, 256, 0, s>>>(pl + 3 * Pl, pl, Pl);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = phys2spec(gl, 6, pl, sg, twl, twl, twl, s);
-    if (e == cudaSuccess) {
-      k_sub<<<blocks(6 * Ml), 256, 0, s>>>(sl, sg, 6 * Ml);
-      e = cudaGetLastError();
-    }
-    // 3. tau = F[uu] - F[ubar ubar]: truncate the difference, back to the LES grid
-    if (e == cudaSuccess) {
-      k_truncate<<<blocks(6 * Ml), 256, 0, s>>>(sl, gl, sg, gl, kc, 6);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = spec2phys(gl, 6, sg, pl, twl, twl, twl, s);
-    if (e == cudaSuccess) {
-      k_rows6<<<bl, 256, 0, s>>>(pl, T, Pl);
-      e = cudaGetLastError();
-    }
-    // 4. features of grad ubar
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sd, uhat_dns, ubytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) {
-      k_truncate<<<blocks(3 * Ml), 256, 0, s>>>(sd, gd, sl, gl, kc, 3);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
-      Spec in;
-      in.p = sl;
-      in.ys = gl.nh;
-      in.zs = (long long)gl.ny * gl.nh;
-      in.cs = (long long)gl.nz * gl.ny * gl.nh;
-      in.zwrap = gl.nz;
-      in.ywrap = gl.ny;
-      Geo gk = gl;
-      gk.Kx = gk.Ky = gk.Kz = kc;
-      k_grad<<<blocks(Ml), 256, 0, s>>>(gk, in, sg);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = spec2phys(gl, 9, sg, pl, twl, twl, twl, s);
-    if (e == cudaSuccess) {
-      k_features<<<bl, 256, 0, s>>>(pl, X, A, Pl, nrm);
-      e = cudaGetLastError();
-    }
+  auto cplx_at = [&](size_t o) { return reinterpret_cast<V*>(base + o); };
+  V *twd = cplx_at(o_twd), *twl = cplx_at(o_twl), *sd = cplx_at(o_sd), *xb = cplx_at(o_xb), *yb = cplx_at(o_yb);
+  V *ub = cplx_at(o_ub), *sl = cplx_at(o_sl), *sg = cplx_at(o_sg);
+  float *pl = reinterpret_cast<float*>(base + o_pl), *nrm = reinterpret_cast<float*>(base + o_nrm);
+  const V* uh = static_cast<const V*>(uhat_dns);
+  const unsigned bl = blocks(Pl);
+  float h[12];
+  for (int i = 0; i < 5; ++i) {
+    h[i] = norm12 ? (float)norm12[i] : 0.f;
+    h[5 + i] = norm12 ? (float)(1.0 / norm12[5 + i]) : 1.f;
   }
-  if (st == PS_OK && e != cudaSuccess) {
+  h[10] = h[11] = 1.f;
+  // backward z and y passes of three fields
+  auto zy = [&](const Geo& g, const V* src, V* dst, const V* tw) {
+    const long long plane = (long long)g.ny * g.nh, fs = (long long)g.nz * plane;
+    const cudaError_t r = c2c(g.nz, +1, src, dst, tw, g.nh, g.ny, fs, g.nh, plane, 3 * g.ny, s);
+    return r != cudaSuccess ? r : c2c(g.ny, +1, dst, dst, tw, g.nh, g.nz, fs, plane, g.nh, 3 * g.nz, s);
+  };
+  cudaError_t e = cudaMemcpyAsync(nrm, h, sizeof(h), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(sl, 0, sizeof(V) * 6 * Ml, s);
+  k_tw<<<(n_dns + 255) / 256, 256, 0, s>>>(twd, n_dns);
+  k_tw<<<(n_les + 255) / 256, 256, 0, s>>>(twl, n_les);
+  // 1. F[u_i u_j], truncated to the LES modes
+  if (e == cudaSuccess) e = zy(gd, uh, sd, twd);
+  if (e == cudaSuccess) e = products(n_dns, sd, xb, yb, sl, twd, kc, n_les, 0, s);
+  // 2. minus F[ubar_i ubar_j]: ubar on the LES grid (kc below 2/3 of the grid,
+  //    so its products do not alias below kc)
+  if (e == cudaSuccess) {
+    k_truncate<<<blocks(3 * Ml), 256, 0, s>>>(uh, gd, ub, gl, kc, 3);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = zy(gl, ub, sg, twl);
+  if (e == cudaSuccess) e = products(n_les, sg, xb, yb, sl, twl, kc, n_les, 1, s);
+  // 3. tau: back to the LES grid
+  if (e == cudaSuccess) e = spec2phys(gl, 6, sl, sl, pl, twl, twl, twl, s);
+  if (e == cudaSuccess) {
+    k_rows6<<<bl, 256, 0, s>>>(pl, T, Pl);
+    e = cudaGetLastError();
+  }
+  // 4. features of grad ubar
+  if (e == cudaSuccess) {
+    Spec in;
+    in.p = ub;
+    in.ys = gl.nh;
+    in.zs = (long long)gl.ny * gl.nh;
+    in.cs = (long long)gl.nz * gl.ny * gl.nh;
+    in.zwrap = gl.nz;
+    in.ywrap = gl.ny;
+    Geo gk = gl;
+    gk.Kx = gk.Ky = gk.Kz = kc;
+    k_grad<<<blocks(Ml), 256, 0, s>>>(gk, in, sg);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = spec2phys(gl, 9, sg, sg, pl, twl, twl, twl, s);
+  if (e == cudaSuccess) {
+    k_features<<<bl, 256, 0, s>>>(pl, X, A, Pl, nrm);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) {
     set_last_error(std::string("ps_les_training_sample: ") + cudaGetErrorString(e));
     st = PS_ERR_CUDA;
   }
   cudaStreamSynchronize(s);
-  for (void* b : bufs) cudaFree(b);
+  cudaFree(base);
   return st;
 }
 
@@ -864,8 +972,7 @@ ps_status fft_run(int n, int nfields, const void* in, void* out, void* cuda_stre
   k_tw<<<(n + 255) / 256, 256, 0, s>>>(tw, n);
   e = cudaGetLastError();
   if (backward) {
-    if (e == cudaSuccess) e = cudaMemcpyAsync(spec, in, sizeof(V) * nfields * M, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = spec2phys(g, nfields, spec, static_cast<float*>(out), tw, tw, tw, s);
+    if (e == cudaSuccess) e = spec2phys(g, nfields, static_cast<const V*>(in), spec, static_cast<float*>(out), tw, tw, tw, s);
   } else {
     if (e == cudaSuccess) e = phys2spec(g, nfields, static_cast<const float*>(in), static_cast<V*>(out), tw, tw, tw, s);
   }
