@@ -114,7 +114,10 @@ void drop_graph(ps_ensemble* e) {
 
 // Sequential: every member's steps on the ensemble stream, member by member.
 ps_status run_sequential(ps_ensemble* e, void* const* u, double dt, double t, int nsteps) {
-  for (size_t i = 0; i < e->plans.size(); ++i) plan_set_stream(e->plans[i], e->main);
+  for (size_t i = 0; i < e->plans.size(); ++i) {
+    plan_set_stream(e->plans[i], e->main);
+    plan_set_beside(e->plans[i], 1);
+  }
   for (int s = 0; s < nsteps; ++s)
     for (size_t i = 0; i < e->plans.size(); ++i) {
       ps_status st = ps_rk_step(e->plans[i], u[i], dt, t + s * dt);
@@ -136,6 +139,7 @@ ps_status capture(ps_ensemble* e, void* const* u, double dt, double t, int nstep
   if (ce != cudaSuccess) st = cu(ce, "fork");
   for (size_t i = 0; i < e->plans.size() && st == PS_OK; ++i) {
     plan_set_stream(e->plans[i], e->branch[i % B]);
+    plan_set_beside(e->plans[i], B);
     plan_invalidate_tables(e->plans[i]);
   }
   for (int s = 0; s < nsteps && st == PS_OK; ++s)

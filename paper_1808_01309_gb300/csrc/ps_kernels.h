@@ -85,6 +85,7 @@ struct PassArgs {
   int Fx, Fy, Fz;
   int xdiag;         // x pass: only the max |u| reduction (no product, no output)
   int xrpc;          // x pass rows per CTA (0 = largest that keeps two CTAs per SM)
+  int beside;        // launches of other plans that run at the same time, this one included (0 = 1)
   int shape[3];      // shape variant of the z-inverse, y and z-forward passes (ColShape; 0 = default)
   int* err;          // device error word (bounded waits that gave up), never null
   unsigned wait_polls;  // x pass: polls before a wait gives up (0 = PS_WAIT_LIMIT)
@@ -172,6 +173,8 @@ cudaError_t les_closure_grad(const Geo& g, Spec in, Spec f, const void* twx, con
 void plan_set_stream(struct ::ps_plan* p, cudaStream_t s);
 cudaStream_t plan_stream(const struct ::ps_plan* p);
 void plan_set_xrpc(struct ::ps_plan* p, int rpc);
+// Launches of other plans that run beside p's, p's included (PassArgs::beside).
+void plan_set_beside(struct ::ps_plan* p, int n);
 // Forget the cached integrating-factor tables so the next step recomputes them
 // (a captured graph must contain that launch).
 void plan_invalidate_tables(struct ::ps_plan* p);

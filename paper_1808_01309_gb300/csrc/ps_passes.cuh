@@ -26,6 +26,8 @@
 
 namespace ps {
 
+constexpr int NSM = 152;  // SMs of a GB300
+
 // kx columns per CTA in the strided passes: 64-byte row segments
 #ifndef PS_TX32
 #define PS_TX32 8
@@ -244,7 +246,13 @@ struct WorkTile {
 
 // One CTA tile (x, y) of the pass; gx = tiles along x (energy partial index
 // y gx + x).  COH: coherent loads (see ldv).
-template <typename T, int N, int NG, int NSC, bool COH, int VAR, class TL>
+//
+// SPLIT: the output fields of a tile are spread over blockIdx.z (zinv_slots):
+// one field per CTA, which stages only the components that field needs (with
+// energy partials the three velocity fields stay together, so the partials are
+// those of the whole tile).
+constexpr int zinv_slots(int ng, int nsc, bool epart) { return ng * (epart ? 4 : 6) + 3 * nsc; }
+template <typename T, int N, int NG, int NSC, bool COH, int VAR, bool SPLIT = false, class TL>
 __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   using V = typename cplx<T>::type;
   using SH = ColShape<T, N, 0, VAR>;
@@ -274,10 +282,24 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   // one group of three components at a time: u (and then B for MHD); then,
   // for the Boussinesq system, the scalar theta (one component) whose
   // gradient i k theta_hat is transformed (three fields)
+  int g0 = 0, g1 = NG + NSC, f0 = 0, f1 = 0, c0 = 0, cstep = 1, nst = 0;
+  if constexpr (SPLIT) {
+    const int per = a.e_part ? 4 : 6, slot = blockIdx.z;
+    g0 = slot < NG * per ? slot / per : NG;
+    g1 = g0 + 1;
+    const int i = slot - g0 * per;  // field (or, with energy partials, the velocity triple first)
+    f0 = a.e_part && g0 < NG ? (i ? i + 2 : 0) : i;
+    f1 = a.e_part && g0 < NG && i == 0 ? 3 : f0 + 1;
+    // components: those of u, or the two of a curl component; theta
+    nst = g0 >= NG ? 1 : f0 >= 3 ? 2 : f1 - f0;
+    c0 = g0 >= NG ? 0 : f0 == 3 ? 1 : f0 > 3 ? 0 : f0;
+    cstep = f0 == 4 ? 2 : 1;
+  }
 #pragma unroll 1
-  for (int grp = 0; grp < NG + NSC; ++grp) {
+  for (int grp = g0; grp < g1; ++grp) {
   const bool sc = grp >= NG;
-  const int ncs = sc ? 1 : 3, nout = sc ? 3 : 6;
+  const int ncs = SPLIT ? nst : sc ? 1 : 3;
+  const int fa = SPLIT ? f0 : 0, fb = SPLIT ? f1 : sc ? 3 : 6;
   const V* in = static_cast<const V*>(a.in.p) + 3 * grp * a.in.cs;
   // stage the tile: element (c, b, i, col) <- u_c(kx0 + col, q_b, r_i) at
   // tile[((c NB + b) cz + i) TX + col]; thread tid keeps column tid % TX and
@@ -302,10 +324,12 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
         if (iyb < g.cy) {
           const int qb = iyb <= g.Ky ? iyb : iyb - g.cy;
           const int r = i <= g.Kz ? i : i - g.cz;
-          const V* src = in + c * a.in.cs + (long long)rowof(r, a.in.zwrap) * a.in.zs +
+          const int cc = SPLIT ? c0 + c * cstep : c;
+          const V* src = in + cc * a.in.cs + (long long)rowof(r, a.in.zwrap) * a.in.zs +
                          (long long)rowof(qb, a.in.ywrap) * a.in.ys + kxc;
-          if constexpr (sizeof(V) == 8) cp_async8(dst, src);
-          else cp_async16(dst, src);
+          V* to = SPLIT ? tile + ((cc * NB + b) * g.cz + i) * TX + col : dst;
+          if constexpr (sizeof(V) == 8) cp_async8(to, src);
+          else cp_async16(to, src);
         }
         i += RSTEP;
         while (i >= g.cz) {
@@ -326,7 +350,7 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   for (int m = 0; m < E; ++m)
     if (bvalid && kx < ncols(g) && kept(g, kxg, q, sidx(j0 + m * (N / E), N))) keepm |= 1u << m;
 #pragma unroll 1
-  for (int f = 0; f < nout; ++f) {
+  for (int f = fa; f < fb; ++f) {
     V x[E];
     T ssq = 0;
 #pragma unroll
@@ -373,16 +397,17 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   }
   __syncthreads();  // the tile is restaged for the next group
   }
-  if (a.e_part) {
+  if (SPLIT ? a.e_part && f0 == 0 : a.e_part != nullptr) {
     // energy 1/2 sum w |u|^2 (+ |B|^2 or theta^2), w = 1 on the kx = 0 plane, else 2
     const double t = block_sum(esum * (kxg == 0 ? 0.5 : 1.0), red);
-    if (threadIdx.x == 0) a.e_part[tl.y() * tl.gx() + tl.x()] = t;
+    const int part = (SPLIT ? g0 * gridDim.y : 0) + tl.y();
+    if (threadIdx.x == 0) a.e_part[part * tl.gx() + tl.x()] = t;
   }
 }
 
-template <typename T, int N, int NG, int NSC, int VAR = 0>
+template <typename T, int N, int NG, int NSC, int VAR = 0, bool SPLIT = false>
 __global__ void __launch_bounds__(ColShape<T, N, 0, VAR>::NTH, MinB<T, N>::zinv) k_zinv(const PassArgs a) {
-  zinv_tile<T, N, NG, NSC, false, VAR>(a, LaunchTile{});
+  zinv_tile<T, N, NG, NSC, false, VAR, SPLIT>(a, LaunchTile{});
 }
 
 // ---------------------------------------------------------------------------
@@ -1016,10 +1041,25 @@ cudaError_t zinv_ng(const PassArgs& a0, cudaStream_t s, int* nb) {
   using SH = ColShape<T, N, 0, VAR>;
   constexpr int TX = SH::TX, NB = SH::NB;
   const size_t smem = (1ull * NB * N * TX + 3ull * NB * a.g.cz * TX) * sizeof(V);
-  cudaError_t e = prep(k_zinv<T, N, NG, NSC, VAR>, smem);
-  if (e != cudaSuccess) return e;
   dim3 grid(a.g.kxp / TX, (a.g.cy + NB - 1) / NB);
   if (nb) *nb = grid.x * grid.y;
+  // A grid of at most two CTAs per SM leaves SMs idle while each CTA transforms
+  // its six fields one after the other: spread the fields over CTAs instead
+  // (64^3 FP32 12.7 -> 5 us a launch).  Not where an ensemble's other members
+  // fill the SMs: there the components staged again cost more than they gain
+  // (48 members: 6.4 ms a step, 7.8 with both this and the smaller row groups).
+  if constexpr (VAR == 0) {
+    if ((long long)grid.x * grid.y * (a.beside ? a.beside : 1) <= 2 * NSM) {
+      cudaError_t e = prep(k_zinv<T, N, NG, NSC, 0, true>, smem);
+      if (e != cudaSuccess) return e;
+      if (nb) *nb *= NG + NSC;
+      grid.z = zinv_slots(NG, NSC, a.e_part != nullptr);
+      k_zinv<T, N, NG, NSC, 0, true><<<grid, SH::NTH, smem, s>>>(a);
+      return cudaGetLastError();
+    }
+  }
+  cudaError_t e = prep(k_zinv<T, N, NG, NSC, VAR>, smem);
+  if (e != cudaSuccess) return e;
   k_zinv<T, N, NG, NSC, VAR><<<grid, SH::NTH, smem, s>>>(a);
   return cudaGetLastError();
 }
@@ -1081,6 +1121,10 @@ cudaError_t xpass_ng(const PassArgs& a0, cudaStream_t s) {
   // rows per CTA: as many as the launch bound allows while two CTAs fit an SM
   int rpc = RPCOf<T, N>::v;
   while (rpc > 1 && xpass_smem<T, N>(a.g, rpc, NF) > 113 * 1024) rpc /= 2;
+  const long long rows = (long long)a.g.nz * a.g.ny;
+  // and fewer (down to a warp's worth) while that leaves SMs without two CTAs
+  const long long beside = a.beside ? a.beside : 1;
+  while (rpc > 1 && rpc * G > 32 && (rows + rpc - 1) / rpc * beside < 2 * NSM) rpc /= 2;
   if (a.xrpc > 0 && a.xrpc < rpc) rpc = a.xrpc;  // tuned (smaller) row groups
   const size_t smem = xpass_smem<T, N>(a.g, rpc, NF);
   cudaError_t e = cudaFuncSetAttribute(k_xpass<T, N, NG, NSC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1091,7 +1135,6 @@ cudaError_t xpass_ng(const PassArgs& a0, cudaStream_t s) {
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_xpass<T, N, NG, NSC>, rpc * G, smem)) !=
       cudaSuccess)
     return e;
-  const long long rows = (long long)a.g.nz * a.g.ny;
   const long long groups = (rows + rpc - 1) / rpc;
   long long grid = (long long)nsm * (per_sm > 0 ? per_sm : 1);
   if (grid > groups) grid = groups;

@@ -144,6 +144,7 @@ struct ps_plan {
   cudaStream_t stream = nullptr;
   int device = 0;
   int xrpc = 0;  // x-pass rows per CTA override (0 = automatic)
+  int beside = 1;            // plans of an ensemble whose launches run at the same time
   int shape[3] = {0, 0, 0};  // shape variants of the z-inverse, y and z-forward passes
   int n_epart_run = 0;       // energy partials written by the last z-inverse launch
   unsigned wait_test_polls = 0;  // ps_plan_set_wait_test: 0 = off
@@ -308,6 +309,7 @@ PassArgs base_args(ps_plan* p) {
   a.acc = p->acc;
   a.err = p->err;
   a.xrpc = p->xrpc;
+  a.beside = p->beside;
   for (int k = 0; k < 3; ++k) a.shape[k] = p->shape[k];
   a.wait_test = p->wait_test_polls ? 1 : 0;
   a.wait_polls = p->wait_test_polls;
@@ -535,6 +537,7 @@ void release(ps_plan* p) {
 namespace ps {
 void plan_set_stream(ps_plan* p, cudaStream_t s) { p->stream = s; }
 cudaStream_t plan_stream(const ps_plan* p) { return p->stream; }
+void plan_set_beside(ps_plan* p, int n) { p->beside = n; }
 void plan_set_xrpc(ps_plan* p, int rpc) {
   if (p->xrpc != rpc) drop_cached_graph(p);
   p->xrpc = rpc;
@@ -671,7 +674,8 @@ ps_status ps_plan_create(const ps_config* cfg, void* cuda_stream, ps_plan** out)
   p->n_epart_run = p->n_epart;
   // room for the partials of every shape variant of the z-inverse pass
   const int nb = f32 ? zinv_blocks<float>(p->g, -1) : zinv_blocks<double>(p->g, -1);
-  ALLOC(p->e_part, sizeof(double) * (size_t)(nb > 0 ? nb : 1), "energy partials");
+  // (one set per field group when the pass spreads the groups over CTAs)
+  ALLOC(p->e_part, sizeof(double) * (size_t)(nb > 0 ? nb : 1) * (p->ng + p->cn.nsc), "energy partials");
   ALLOC(p->stats, sizeof(double) * 4, "stats");
   ALLOC(p->umax2, sizeof(unsigned long long), "max|u|");
   ALLOC(p->ext, sizeof(int) * 4, "forcing extent");
