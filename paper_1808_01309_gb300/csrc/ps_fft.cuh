@@ -240,6 +240,7 @@ template <> struct Sched<128, 8> { static constexpr int S = 3, R0 = 8, R1 = 8, R
 template <> struct Sched<256, 16> { static constexpr int S = 2, R0 = 16, R1 = 16, R2 = 1, R3 = 1; };
 template <> struct Sched<256, 8> { static constexpr int S = 3, R0 = 8, R1 = 8, R2 = 4, R3 = 1; };
 template <> struct Sched<512, 8> { static constexpr int S = 3, R0 = 8, R1 = 8, R2 = 8, R3 = 1; };
+template <> struct Sched<512, 16> { static constexpr int S = 3, R0 = 16, R1 = 16, R2 = 2, R3 = 1; };
 template <> struct Sched<1024, 16> { static constexpr int S = 3, R0 = 16, R1 = 8, R2 = 8, R3 = 1; };
 template <> struct Sched<1024, 8> { static constexpr int S = 4, R0 = 8, R1 = 8, R2 = 8, R3 = 2; };
 // lengths with a factor 3 (E = 12)
@@ -570,6 +571,53 @@ __device__ __forceinline__ void fx_row_bounds(int (&u)[NL], X& ex) {
   }
 }
 
+// Where element m of thread j0 lies on its line, before and after line_fft.
+template <typename T, int N, int E> struct LinePos {
+  static constexpr bool paired = sizeof(T) == 4 && N == 512 && E == 16;
+  __device__ static __forceinline__ int in(int j0, int m) { return j0 + m * (N / E); }
+  __device__ static __forceinline__ int out(int j0, int m) {
+    if constexpr (paired) return (j0 >> 1) + 128 * (j0 & 1) + 16 * (m & 7) + 256 * (m >> 3);
+    else return in(j0, m);
+  }
+};
+
+// A 512-point FP32 column line over 32 threads of 16 points: thread j0 = 2 k + h
+// holds the elements j0 + 32 m, threads of one h transform the even or odd
+// elements as 256 = 16 x 16 points (one exchange), and a radix-2 step with the
+// neighbour j0 ^ 1 (TX lanes away: shuffles) completes the line.  The odd inputs
+// of the second radix-16 step change sign where h = 1, which swaps its output
+// halves: a[r] is what the thread keeps, a[r + 8] what its neighbour needs.
+// Three radix-8 stages over 64 threads (two exchanges, each behind two CTA-wide
+// barriers) took longer in every strided pass (ps_passes.cuh).  The caller
+// synchronises before the exchange buffer is used again.
+template <int DIR, int TX, class X>
+__device__ __forceinline__ void line_fft_paired(float2 (&a)[16], int j0, const float2* __restrict__ tw, X& ex) {
+  const int k = j0 >> 1, h = j0 & 1;
+  dft<16, DIR>(a);
+  float2* b = ex.buf + h * TX + ex.l;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) b[2 * TX * (16 * k + r)] = a[r];
+  ex.sync();
+#pragma unroll
+  for (int r = 0; r < 16; ++r) a[r] = b[2 * TX * (k + 16 * r)];
+#pragma unroll
+  for (int r = 1; r < 16; ++r) {
+    const float2 w = __ldg(tw + ((2 * r * k + (r & 1) * 256 * h) & 511));
+    a[r] = cmul(a[r], DIR > 0 ? cconj(w) : w);
+  }
+  dft<16, DIR>(a);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, a[r + 8].x, TX),
+                                   __shfl_xor_sync(0xffffffffu, a[r + 8].y, TX));
+    const float2 ev = make_float2(h ? got.x : a[r].x, h ? got.y : a[r].y);
+    const float2 w = __ldg(tw + k + 128 * h + 16 * r);
+    const float2 od = cmul(make_float2(h ? a[r].x : got.x, h ? a[r].y : got.y), DIR > 0 ? cconj(w) : w);
+    a[r] = cadd(ev, od);
+    a[r + 8] = csub(ev, od);
+  }
+}
+
 // Full length-N transform of a column line with twiddles read from global
 // memory (FP64: in block fixed point, ps_fix.cuh).
 template <int N, int E, int DIR, typename V, class X>
@@ -584,6 +632,8 @@ __device__ __forceinline__ void line_fft(V (&a)[E], int j0, const void* twp, X& 
     line_fft_tw<N, E, DIR>(b, j0, tw, ex);
 #pragma unroll
     for (int m = 0; m < E; ++m) a[m] = fx_value(b[m], sc);
+  } else if constexpr (LinePos<float, N, E>::paired) {
+    line_fft_paired<DIR, X::cols>(a, j0, tw.p, ex);
   } else {
     line_fft_tw<N, E, DIR>(a, j0, tw, ex);
   }

@@ -44,7 +44,7 @@ template <typename T, int K = 0> struct TXOf {
 // against 13.08 ms at 8 points per thread (four stages, three exchanges)
 // and 14.70 ms at 16 points capped to 128 registers (spills).
 template <typename T, int N, int K> struct EPass {
-  static constexpr int v = EOf<T, N>::v;
+  static constexpr int v = sizeof(T) == 4 && N == 512 && (K == 1 || K == 2) ? 16 : EOf<T, N>::v;
 };
 // lines batched per CTA in the strided passes (about 256 threads per CTA)
 template <typename T, int N, int K = 0> struct NBOf {
@@ -390,10 +390,11 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
     if (bvalid) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
-        const int n = j0 + m * (N / E);
+        const int n = LinePos<T, N, E>::out(j0, m);
         out[(6 * grp + f) * fstride + n * zstride + (long long)iy * g.kxp + kx] = x[m];
       }
     }
+    if constexpr (LinePos<T, N, E>::paired) __syncthreads();  // the exchange buffer is free again
   }
   __syncthreads();  // the tile is restaged for the next group
   }
@@ -443,7 +444,7 @@ __device__ __forceinline__ void yinv_tile(const PassArgs& a, const TL& tl) {
   line_fft<N, E, +1>(x, j0, a.tw_y, ex);
   if (bvalid) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) out[(long long)(j0 + m * (N / E)) * g.kxp] = x[m];
+    for (int m = 0; m < E; ++m) out[(long long)LinePos<T, N, E>::out(j0, m) * g.kxp] = x[m];
   }
 }
 
@@ -771,7 +772,7 @@ __device__ __forceinline__ void yfwd_tile(const PassArgs& a, const TL& tl) {
   if (bvalid) {
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const int q = sidx(j0 + m * (N / E), N);
+      const int q = sidx(LinePos<T, N, E>::out(j0, m), N);
       if (q <= g.Ky && q >= -g.Ky) out[(long long)rowof(q, g.cy) * g.kxp] = x[m];
     }
   }
@@ -817,7 +818,7 @@ __device__ __forceinline__ void zfwd_tile(const PassArgs& a, const TL& tl) {
     V* out = static_cast<V*>(a.a6) + (long long)f * g.cz * g.cy * g.kxp + (long long)iy * g.kxp + kx;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const int r = sidx(j0 + m * (N / E), N);
+      const int r = sidx(LinePos<T, N, E>::out(j0, m), N);
       if (r <= g.Kz && r >= -g.Kz)
         out[(long long)rowof(r, g.cz) * g.cy * g.kxp] =
             kx < ncols(g) && kept(g, g.kx0 + kx, q, r) ? cscale(x[m], inv) : czero<V>();
