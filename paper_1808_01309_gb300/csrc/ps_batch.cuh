@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v), MinB
   const long long total = ng * M;
   V* stage = reinterpret_cast<V*>(smraw);
   V* exbuf = stage + NF * rpc * kxp;
-  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLINES * N, N, 0, 0};
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLines<T, N>::v * N, N, 0, 0};
   if (G >= 32) {
     ex.bar_id = 1 + rl;
     ex.nthr = G;
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v), MinB
   if constexpr (TR) {
     tw.load(static_cast<const W*>(B.args[0].tw_x), j0);
   } else if constexpr (TT) {
-    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLINES * N);
+    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLines<T, N>::v * N);
     if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const W*>(B.args[0].tw_x), j0);
     tw = TwAcc{twt, j0};
   } else {

@@ -525,19 +525,19 @@ struct LinesExchange {
   }
 };
 
-// Bound of sum |re| + |im| over the line from its threads' parts u, for lines
+// Bound of sum |re| + |im| over a line from its threads' elements, for lines
 // laid out as columns: TX lines side by side, thread = line + TX (j0 + G b).
 // Every thread of the CTA calls it; the lines of a CTA exchange at least once
 // between two calls, so the shared words of a call are read before the next
 // call writes them.
-template <int TX, int G>
-__device__ __forceinline__ int fx_column_bound(int u) {
+template <int TX, int G, int E>
+__device__ __forceinline__ int fx_column_bound(const double2 (&a)[E]) {
   if constexpr (TX * G <= 32) {
-    return fx_lane_sum<TX, TX * G>(u);
+    return fx_bound<TX, TX * G>(a);
   } else {
     constexpr int W = TX * G / 32;  // warps of a line
     __shared__ int part[32 * TX];
-    u = fx_lane_sum<TX, 32>(u);
+    int u = fx_bound<TX, 32>(a);
     const int w = threadIdx.x >> 5, l = threadIdx.x % TX;
     if ((threadIdx.x & 31) < TX) part[w * TX + l] = u;
     __syncthreads();
@@ -548,27 +548,21 @@ __device__ __forceinline__ int fx_column_bound(int u) {
     return u;
   }
 }
-// The same for the NL lines of a row spread over G consecutive threads.
-template <int G, int NL, class X>
-__device__ __forceinline__ void fx_row_bounds(int (&u)[NL], X& ex) {
-#pragma unroll
-  for (int l = 0; l < NL; ++l) u[l] = fx_lane_sum<1, (G < 32 ? G : 32)>(u[l]);
+// The same for a row spread over G consecutive threads.
+template <int G, int E, class X>
+__device__ __forceinline__ int fx_row_bound(const double2 (&a)[E], X& ex) {
+  int u = fx_bound<1, (G < 32 ? G : 32)>(a);
   if constexpr (G > 32) {
     constexpr int W = G / 32;
-    __shared__ int part[32 * 3];
-    static_assert(NL <= 3, "lines of a row transformed together");
+    __shared__ int part[32];
     const int w = threadIdx.x >> 5, w0 = w / W * W;
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-      for (int l = 0; l < NL; ++l) part[w * 3 + l] = u[l];
+    if ((threadIdx.x & 31) == 0) part[w] = u;
     ex.sync();
+    u = part[w0];
 #pragma unroll
-    for (int l = 0; l < NL; ++l) {
-      u[l] = part[w0 * 3 + l];
-#pragma unroll
-      for (int i = 1; i < W; ++i) u[l] = fx_add_bound(u[l], part[(w0 + i) * 3 + l]);
-    }
+    for (int i = 1; i < W; ++i) u = fx_add_bound(u, part[w0 + i]);
   }
+  return u;
 }
 
 // Where element m of thread j0 lies on its line, before and after line_fft.
@@ -626,7 +620,7 @@ __device__ __forceinline__ void line_fft(V (&a)[E], int j0, const void* twp, X& 
   const GlobalTw<W> tw{static_cast<const W*>(twp)};
   if constexpr (std::is_same<V, double2>::value) {
     static_assert(X::cols > 0, "columns of the tile");
-    const FxScale sc = fx_scale(fx_column_bound<X::cols, N / E>(fx_partial(a)));
+    const FxScale sc = fx_scale(fx_column_bound<X::cols, N / E>(a));
     fx2 b[E];
     fx_load(b, a, sc);
     line_fft_tw<N, E, DIR>(b, j0, tw, ex);
@@ -708,49 +702,30 @@ __device__ __forceinline__ void line_fft_rows(V (&a)[NL][E], int j0, const TW& t
   }
 }
 
-// The lines before and after line_fft_rows: FP32 values as they are; FP64
-// values in block fixed point, with the scale of each line.
-template <int N, int E, int NL, class X>
-__device__ __forceinline__ void rows_load(float2 (&b)[NL][E], const float2 (&a)[NL][E], FxScale (&)[NL], X&) {
-#pragma unroll
-  for (int l = 0; l < NL; ++l)
-#pragma unroll
-    for (int m = 0; m < E; ++m) b[l][m] = a[l][m];
+// Transform of NL lines of a row in place: FP32 lines together (one exchange
+// for all of them); FP64 lines one after the other, through block fixed point,
+// which leaves registers and shared memory for more rows per SM.
+template <int N, int E, int DIR, int NL, class TW, class X>
+__device__ __forceinline__ void rows_fft(float2 (&a)[NL][E], int j0, const TW& tw, X& ex) {
+  line_fft_rows<N, E, DIR>(a, j0, tw, ex);
 }
-template <int N, int E, int NL, class X>
-__device__ __forceinline__ void rows_load(fx2 (&b)[NL][E], const double2 (&a)[NL][E], FxScale (&sc)[NL], X& ex) {
-  int u[NL];
-#pragma unroll
-  for (int l = 0; l < NL; ++l) u[l] = fx_partial(a[l]);
-  fx_row_bounds<N / E>(u, ex);
+// One FP64 line into fixed point and through the transform; returns its scale.
+template <int N, int E, int DIR, class TW, class X>
+__device__ __forceinline__ FxScale row_fft_fix(fx2 (&b)[1][E], const double2 (&a)[E], int j0, const TW& tw, X& ex) {
+  const FxScale sc = fx_scale(fx_row_bound<N / E>(a, ex));
+  fx_load(b[0], a, sc);
+  line_fft_rows<N, E, DIR>(b, j0, tw, ex);
+  return sc;
+}
+template <int N, int E, int DIR, int NL, class TW, class X>
+__device__ __forceinline__ void rows_fft(double2 (&a)[NL][E], int j0, const TW& tw, X& ex) {
 #pragma unroll
   for (int l = 0; l < NL; ++l) {
-    sc[l] = fx_scale(u[l]);
-    fx_load(b[l], a[l], sc[l]);
+    fx2 b[1][E];
+    const FxScale sc = row_fft_fix<N, E, DIR>(b, a[l], j0, tw, ex);
+#pragma unroll
+    for (int m = 0; m < E; ++m) a[l][m] = fx_value(b[0][m], sc);
   }
-}
-// One value of a transformed line, halved if HALF.
-template <bool HALF = false>
-__device__ __forceinline__ float2 line_value(float2 v, FxScale) {
-  if constexpr (HALF) return cscale(v, 0.5f);
-  return v;
-}
-template <bool HALF = false>
-__device__ __forceinline__ double2 line_value(fx2 v, FxScale sc) {
-  if constexpr (HALF) sc.s += 1;
-  return fx_value(v, sc);
-}
-// Transform of NL lines in place.
-template <int N, int E, int DIR, int NL, typename V, class TW, class X>
-__device__ __forceinline__ void rows_fft(V (&a)[NL][E], int j0, const TW& tw, X& ex) {
-  typename fft_of<V>::val b[NL][E];
-  FxScale sc[NL];
-  rows_load<N>(b, a, sc, ex);
-  line_fft_rows<N, E, DIR>(b, j0, tw, ex);
-#pragma unroll
-  for (int l = 0; l < NL; ++l)
-#pragma unroll
-    for (int m = 0; m < E; ++m) a[l][m] = line_value(b[l][m], sc[l]);
 }
 
 }  // namespace ps

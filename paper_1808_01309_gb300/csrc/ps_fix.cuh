@@ -172,17 +172,30 @@ __host__ __device__ __forceinline__ void fx_to(long long v, FxScale f, int& hi, 
 }
 
 #ifdef __CUDACC__
-// High word of an upper bound of sum |re| + |im| over E elements (0 when all
-// are zero or subnormal, the high word of Inf or more for an Inf or NaN): the
-// terms as FP32 numbers relative to the largest exponent.
-template <int E>
-__device__ __forceinline__ int fx_partial(const double2 (&a)[E]) {
+// v over the lanes lane ^ FROM, ^ 2 FROM, ... below WIDTH: every lane of the
+// aligned group of WIDTH lanes gets the same largest value or sum.
+template <int FROM, int WIDTH, class V, class OP>
+__device__ __forceinline__ V fx_lanes(V v, OP op) {
+  unsigned mask = 0xffffffffu;
+  if constexpr (WIDTH < 32) mask = ((1u << WIDTH) - 1u) << (threadIdx.x & 31 & ~(WIDTH - 1));
+#pragma unroll
+  for (int o = FROM; o < WIDTH; o *= 2) v = op(v, __shfl_xor_sync(mask, v, o));
+  return v;
+}
+// High word of an upper bound of sum |re| + |im| over the E elements of each
+// lane of such a group (0 when all are zero or subnormal, that of Inf for an Inf
+// or NaN).  The terms are added as FP32 numbers relative to the largest exponent
+// of the group: FP64 additions would take the pipe this format avoids.
+template <int FROM, int WIDTH, int E>
+__device__ __forceinline__ int fx_bound(const double2 (&a)[E]) {
   int hm = 0;
 #pragma unroll
   for (int m = 0; m < E; ++m) {
     hm = max(hm, __double2hiint(a[m].x) & 0x7fffffff);
     hm = max(hm, __double2hiint(a[m].y) & 0x7fffffff);
   }
+  if constexpr (FROM == 1 && WIDTH == 32) hm = __reduce_max_sync(0xffffffffu, hm);
+  else hm = fx_lanes<FROM, WIDTH>(hm, [](int x, int y) { return max(x, y); });
   const int base = (hm & 0x7ff00000) - (127 << 20);
   float f = 0.f;
 #pragma unroll
@@ -190,7 +203,8 @@ __device__ __forceinline__ int fx_partial(const double2 (&a)[E]) {
     f += __int_as_float(max((__double2hiint(a[m].x) & 0x7fffffff) - base, 0) << 3);
     f += __int_as_float(max((__double2hiint(a[m].y) & 0x7fffffff) - base, 0) << 3);
   }
-  // truncated terms (2^-20 of each) and the FP32 sum: raised by 2^-9
+  f = fx_lanes<FROM, WIDTH>(f, [](float x, float y) { return x + y; });
+  // truncated terms (2^-20 of each) and the FP32 sums: raised by 2^-9
   const unsigned u = (unsigned)((__float_as_int(f) >> 3) + base + (1 << 11));
   return hm < 0x00100000 ? 0 : (int)min(u, 0x7ff00000u);
 }
@@ -198,16 +212,6 @@ __device__ __forceinline__ int fx_partial(const double2 (&a)[E]) {
 __device__ __forceinline__ int fx_add_bound(int u, int v) {
   const unsigned w = (unsigned)__double2hiint(__hiloint2double(u, 0) + __hiloint2double(v, 0)) + 1u;
   return (int)min(w, 0x7ff00000u);
-}
-// Sum over the lanes lane ^ FROM, ^ 2 FROM, ... below WIDTH; every lane of the
-// aligned group of WIDTH lanes holds the same value.
-template <int FROM, int WIDTH>
-__device__ __forceinline__ int fx_lane_sum(int u) {
-  unsigned mask = 0xffffffffu;
-  if constexpr (WIDTH < 32) mask = ((1u << WIDTH) - 1u) << (threadIdx.x & 31 & ~(WIDTH - 1));
-#pragma unroll
-  for (int o = FROM; o < WIDTH; o *= 2) u = fx_add_bound(u, __shfl_xor_sync(mask, u, o));
-  return u;
 }
 template <int E>
 __device__ __forceinline__ void fx_load(fx2 (&b)[E], const double2 (&a)[E], FxScale f) {

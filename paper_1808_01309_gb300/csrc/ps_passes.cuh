@@ -78,20 +78,33 @@ template <typename T, int N> struct HasShapes {
   static constexpr bool v = sizeof(T) == 4 && (N == 64 || N == 96 || N == 128);
 };
 
+// x pass: lines per row transformed together (exchange region of a row).  The
+// FP32 hydrodynamic rows take three; the others one line at a time: with three,
+// registers and shared memory held the SM to eight warps (FP64), or six (MHD at
+// 256 points).
+#ifndef PS_XSEQ
+#define PS_XSEQ 0
+#endif
+#ifndef PS_XSEQB
+#define PS_XSEQB 3
+#endif
+template <typename T, int N, bool HD = true> struct XLines {
+  static constexpr int v = sizeof(T) == 4 && HD && !PS_XSEQ ? 3 : 1;
+};
+
 // rows per CTA in the x pass
-template <typename T, int N> struct RPCOf {
+template <typename T, int N, bool HD = true> struct RPCOf {
   static constexpr int G = N / EPass<T, N, 3>::v;
-  static constexpr int v = G >= 256 ? 1 : 256 / G;
+  static constexpr int NT = XLines<T, N, HD>::v == 3 ? 256 : 128;  // threads per CTA
+  static constexpr int v = G >= NT ? 1 : NT / G;
 };
 
 // x pass: per-thread twiddle table in shared memory when it takes at most 8 KB
+// (16 KB in FP64)
 template <typename T, int N> struct XTwTable {
   static constexpr int E = EPass<T, N, 3>::v;
-  static constexpr bool v = (size_t)TwSlots<N, E>::total * (N / E) * sizeof(typename cplx<T>::type) <= 8192;
+  static constexpr bool v = (size_t)TwSlots<N, E>::total * (N / E) * sizeof(typename cplx<T>::type) <= (sizeof(T) == 8 ? 16384 : 8192);
 };
-
-// x pass: lines per row transformed together (exchange region of a row)
-constexpr int XLINES = 3;
 
 // x pass: twiddles in registers for the whole kernel when there are few
 #ifndef PS_XTWREG
@@ -111,6 +124,9 @@ template <typename T, int N> struct XTwReg {
 #endif
 #ifndef PS_MINB_XPASS
 #define PS_MINB_XPASS 2
+#endif
+#ifndef PS_MINB_X64
+#define PS_MINB_X64 3
 #endif
 #ifndef PS_MINB_Y1024
 #define PS_MINB_Y1024 2
@@ -155,13 +171,16 @@ template <typename T, int N> struct XHalved {
   static constexpr int E = EPass<T, N, 3>::v, R = RPCOf<T, N>::v;
   static constexpr long long tt =
       (!XTwReg<T, N>::v && XTwTable<T, N>::v) ? (long long)TwSlots<N, E>::total * (N / E) : 0;
-  static constexpr long long bytes = (6LL * R * kxp + 3LL * R * N + tt) * (long long)sizeof(typename cplx<T>::type);
+  static constexpr long long bytes =
+      (6LL * R * kxp + (long long)XLines<T, N>::v * R * N + tt) * (long long)sizeof(typename cplx<T>::type);
   static constexpr bool v = bytes > 113LL * 1024;
 };
 template <typename T, int N> struct MinB {
   // (1024-point z lines: the input tile and exchange hold one CTA per SM)
   static constexpr int zinv = N == 1024 ? 1 : PS_MINB_ZINV;
-  static constexpr int xpass = XHalved<T, N>::v ? 1 : PS_MINB_XPASS;
+  // x pass with two groups or a scalar: 96 to 192 registers hold the packed lines
+  static constexpr int xmulti = sizeof(T) == 4 && EPass<T, N, 3>::v == 8 ? 3 : 2;
+  static constexpr int xpass = XLines<T, N>::v == 1 && sizeof(T) == 4 ? PS_XSEQB : sizeof(T) == 8 ? (N == 1024 || N % 3 == 0 ? 2 : PS_MINB_X64) : XHalved<T, N>::v ? 1 : PS_MINB_XPASS;
   static constexpr int ypass = sizeof(T) == 4 && N == 1024 ? PS_MINB_Y1024 : sizeof(T) == 4 && N == 512 ? PS_MINB_Y512 : 0;
   static constexpr int zfwd = sizeof(T) == 4 && N == 1024 ? PS_MINB_ZF1024 : sizeof(T) == 4 && N == 512 ? PS_MINB_ZF512 : 0;
 };
@@ -466,6 +485,101 @@ __global__ void __launch_bounds__(ColShape<T, N, 1, VAR>::NTH, MinB<T, N>::ypass
 // NSC = 1 (Boussinesq): u + i omega and grad theta in, u x omega and
 // u . grad theta out.
 // ---------------------------------------------------------------------------
+// The FP64 hydrodynamic row: its five lines one after the other through one copy
+// of the fixed-point transform (a forward line as the backward transform of the
+// swapped values, swapped back).  With the five transforms written out the
+// kernel overran the instruction cache (ncu: no_instruction 1.8 of 9.9 stalls
+// per issue).
+template <int N, int E, bool COH, class TW, class AfterGather>
+__device__ __forceinline__ void xpass_row_fix(const PassArgs& a, const long long row, const bool rvalid, const int j0,
+                                              const double2* st, const long long fst, const TW& tw,
+                                              LinesExchange<fx2, 1>& ex, double& umax2, AfterGather&& gathered) {
+  using V = double2;
+  const Geo& g = a.g;
+  const int kxp = g.kxp;
+  const long long rows = (long long)g.nz * g.ny, rrow = rvalid ? row : 0;
+  const int kend = kxp < N / 2 + 1 ? kxp : N / 2 + 1;
+  V U[2][E];  // u_c + i omega_c of the last two lines at the thread's points; then n_z in U[0][.].x
+  V x[E];     // the line to transform
+#pragma unroll 1
+  for (int job = 0; job < 5; ++job) {
+    if (job < 3) {
+      const V* pu = st + job * fst;
+      const V* pw = st + (job + 3) * fst;
+#pragma unroll
+      for (int m = 0; m < E; ++m) {
+        const int n = j0 + m * (N / E);
+        const bool hi = n > N / 2;  // (as in xpass_row)
+        const int p = hi ? N - n : n;
+        V v = czero<V>();
+        if (rvalid && p <= g.Kx) {
+          V X = COH ? ldv<true>(pu + p) : pu[p], W = COH ? ldv<true>(pw + p) : pw[p];
+          if (hi) {
+            X = cconj(X);
+            W = cconj(W);
+          }
+          v = mk<V>(X.x - W.y, X.y + W.x);
+        }
+        x[m] = v;
+      }
+      if (job == 2) gathered();
+    } else if (job == 4) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) x[m] = mk<V>(0.0, U[0][m].x);
+    }
+    fx2 b[1][E];
+    FxScale sc = row_fft_fix<N, E, +1>(b, x, j0, tw, ex);
+    if (job < 2) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) {
+        U[0][m] = U[1][m];
+        U[1][m] = fx_value(b[0][m], sc);
+      }
+      continue;
+    }
+    if (job == 2) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) {
+        const V v = fx_value(b[0][m], sc);
+        const double ux = U[0][m].x, uy = U[1][m].x, uz = v.x, wx = U[0][m].y, wy = U[1][m].y, wz = v.y;
+        if (a.umax2) umax2 = fmax(umax2, ux * ux + uy * uy + uz * uz);
+        x[m] = mk<V>(uz * wx - ux * wz, uy * wz - uz * wy);  // n_x + i n_y, swapped
+        U[0][m].x = ux * wy - uy * wx;
+      }
+      if (a.xdiag) return;  // uniform across the grid
+      continue;
+    }
+    // n_x and n_y split with the mirrored entry, or n_z as it is
+    V* ca = static_cast<V*>(a.a6) + ((long long)(job == 3 ? 0 : 2) * rows + rrow) * kxp;
+    V* cb = ca + rows * kxp;
+    if (job == 3) {
+      sc.s += 1;  // the split's factor 1/2
+#pragma unroll
+      for (int m = 0; m < E; ++m) ex.template put<0, 0>(0, j0 + m * (N / E), b[0][m]);
+      ex.sync();
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int k = j0 + m * (N / E);
+      if (rvalid && k < kend) {
+        V va = czero<V>(), vb = va;
+        if (k <= g.Kx) {
+          fx2 f = mk<fx2>(b[0][m].y, b[0][m].x);
+          if (job == 3) {
+            const fx2 t = ex.template get<0, 0>(0, k == 0 ? 0 : N - k), fm = mk<fx2>(t.y, -t.x);
+            vb = fx_value(cmul_mi(csub(f, fm)), sc);
+            f = cadd(f, fm);
+          }
+          va = fx_value(f, sc);
+        }
+        ca[k] = va;
+        if (job == 3) cb[k] = vb;
+      }
+    }
+    if (job == 3) ex.sync();
+  }
+}
+
 // The work of the x pass on one row: gather the packed inverse lines (field f
 // of the row at st + f fst, retained kx only), transform them, form the
 // products, transform forward, split and store the retained kx of the output
@@ -487,6 +601,9 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
   const int kxp = g.kxp;
   const long long rows = (long long)g.nz * g.ny;
   V* C = static_cast<V*>(a.a6);
+  if constexpr (sizeof(T) == 8 && HD) {
+    xpass_row_fix<N, E, COH>(a, row, rvalid, j0, st, fst, tw, ex, umax2, gathered);
+  } else {
   // packed lines: u_c + i omega_c (c < 3) and, for MHD, B_c + i j_c; for
   // the Boussinesq system d_x theta + i d_y theta and d_z theta + i 0
   V U[NLI][E];
@@ -525,41 +642,19 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
     }
   }
   gathered();
-  if constexpr (HD) {
+  constexpr bool SEQ = XLines<T, N, HD>::v == 1;  // one line after the other
+  if constexpr (!SEQ) {
     rows_fft<N, E, +1>(U, j0, tw, ex);
-  } else if constexpr (NSC == 1) {
-    V L[3][E], S[2][E];
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int m = 0; m < E; ++m) L[c][m] = U[c][m];
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-      for (int m = 0; m < E; ++m) S[c][m] = U[3 + c][m];
-    rows_fft<N, E, +1>(L, j0, tw, ex);
-    rows_fft<N, E, +1>(S, j0, tw, ex);
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int m = 0; m < E; ++m) U[c][m] = L[c][m];
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-      for (int m = 0; m < E; ++m) U[3 + c][m] = S[c][m];
   } else {
+    // one line after the other
 #pragma unroll
-    for (int h = 0; h < NG; ++h) {
-      V L[3][E];
+    for (int c = 0; c < NLI; ++c) {
+      V L[1][E];
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int m = 0; m < E; ++m) L[c][m] = U[3 * h + c][m];
+      for (int m = 0; m < E; ++m) L[0][m] = U[c][m];
       rows_fft<N, E, +1>(L, j0, tw, ex);
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int m = 0; m < E; ++m) U[3 * h + c][m] = L[c][m];
+      for (int m = 0; m < E; ++m) U[c][m] = L[0][m];
     }
   }
   // products at the thread's points (real part = field, imaginary = curl)
@@ -568,7 +663,7 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
   for (int m = 0; m < E; ++m) {
     const T ux = U[0][m].x, uy = U[1][m].x, uz = U[2][m].x;
     const T wx = U[0][m].y, wy = U[1][m].y, wz = U[2][m].y;
-    umax2 = fmax(umax2, ux * ux + uy * uy + uz * uz);
+    if (sizeof(T) == 4 || a.umax2) umax2 = fmax(umax2, ux * ux + uy * uy + uz * uz);
     T nx = uy * wz - uz * wy, ny = uz * wx - ux * wz, nz = ux * wy - uy * wx;
     if constexpr (HD) {
       F[0][m] = mk<V>(nx, ny);
@@ -591,53 +686,123 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
     }
   }
   if (!a.xdiag) {  // uniform across the grid
-    using FV = typename fft_of<V>::val;
-    FV H[NFW][E];
-    FxScale sc[NFW];
-    rows_load<N>(H, F, sc, ex);
-    line_fft_rows<N, E, -1>(H, j0, tw, ex);
     const long long rrow = rvalid ? row : 0;
     const int kend = kxp < N / 2 + 1 ? kxp : N / 2 + 1;
     // split each packed transform F = DFT(a) + i DFT(b) of two real fields
-    // with its mirrored entry F[N-k] (all split lines through one exchange);
-    // for HD the second line has b = 0
+    // with its mirrored entry F[N-k]; for HD the second line has b = 0
     constexpr int NSP = HD ? 1 : NFW;  // lines that need the split
+    if constexpr (!HD && sizeof(T) == 8) {
+      // one line after the other, split in fixed point
 #pragma unroll
-    for (int w = 0; w < NSP; ++w)
+      for (int w = 0; w < NFW; ++w) {
+        fx2 H[1][E];
+        FxScale sc = row_fft_fix<N, E, -1>(H, F[w], j0, tw, ex);
+        const bool split = w < NSP;
+        if (split) {
+          sc.s += 1;  // the split's factor 1/2
 #pragma unroll
-      for (int m = 0; m < E; ++m) ex.template put<0, 0>(w, j0 + m * (N / E), H[w][m]);
-    ex.sync();
+          for (int m = 0; m < E; ++m) ex.template put<0, 0>(0, j0 + m * (N / E), H[0][m]);
+          ex.sync();
+        }
+        V* ca = C + ((long long)(2 * w) * rows + rrow) * kxp;
+        V* cb = C + ((long long)(2 * w + 1) * rows + rrow) * kxp;
 #pragma unroll
-    for (int w = 0; w < NFW; ++w) {
-      const bool split = w < NSP;
-      V* ca = C + ((long long)(2 * w) * rows + rrow) * kxp;
-      V* cb = C + ((long long)(2 * w + 1) * rows + rrow) * kxp;
-#pragma unroll
-      for (int m = 0; m < E; ++m) {
-        const int k = j0 + m * (N / E);
-        if (rvalid && k < kend) {
-          V va = czero<V>(), vb = czero<V>();
-          if (k <= g.Kx) {
-            const FV Fk = H[w][m];
-            if (split) {
-              const FV Fm = cconj(ex.template get<0, 0>(w, k == 0 ? 0 : N - k));
-              va = line_value<true>(cadd(Fk, Fm), sc[w]);
-              vb = line_value<true>(cmul_mi(csub(Fk, Fm)), sc[w]);
-            } else {
-              va = line_value(Fk, sc[w]);
+        for (int m = 0; m < E; ++m) {
+          const int k = j0 + m * (N / E);
+          if (rvalid && k < kend) {
+            V va = czero<V>(), vb = czero<V>();
+            if (k <= g.Kx) {
+              if (split) {
+                const fx2 Fm = cconj(ex.template get<0, 0>(0, k == 0 ? 0 : N - k));
+                va = fx_value(cadd(H[0][m], Fm), sc);
+                vb = fx_value(cmul_mi(csub(H[0][m], Fm)), sc);
+              } else {
+                va = fx_value(H[0][m], sc);
+              }
             }
+            ca[k] = va;
+            if (split) cb[k] = vb;
           }
-          ca[k] = va;
-          if (split) cb[k] = vb;
+        }
+        if (split && w + 1 < NFW) ex.sync();
+      }
+    } else if constexpr (SEQ) {
+      // one line after the other
+#pragma unroll
+      for (int w = 0; w < NFW; ++w) {
+        V H[1][E];
+#pragma unroll
+        for (int m = 0; m < E; ++m) H[0][m] = F[w][m];
+        line_fft_rows<N, E, -1>(H, j0, tw, ex);
+        const bool split = w < NSP;
+        if (split) {
+#pragma unroll
+          for (int m = 0; m < E; ++m) ex.template put<0, 0>(0, j0 + m * (N / E), H[0][m]);
+          ex.sync();
+        }
+        V* ca = C + ((long long)(2 * w) * rows + rrow) * kxp;
+        V* cb = C + ((long long)(2 * w + 1) * rows + rrow) * kxp;
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+          const int k = j0 + m * (N / E);
+          if (rvalid && k < kend) {
+            V va = czero<V>(), vb = czero<V>();
+            if (k <= g.Kx) {
+              if (split) {
+                const V Fm = cconj(ex.template get<0, 0>(0, k == 0 ? 0 : N - k));
+                va = cscale(cadd(H[0][m], Fm), T(0.5));
+                vb = cscale(cmul_mi(csub(H[0][m], Fm)), T(0.5));
+              } else {
+                va = H[0][m];
+              }
+            }
+            ca[k] = va;
+            if (split) cb[k] = vb;
+          }
+        }
+        if (split && w + 1 < NFW) ex.sync();
+      }
+    } else {
+      line_fft_rows<N, E, -1>(F, j0, tw, ex);
+      // all split lines through one exchange
+#pragma unroll
+      for (int w = 0; w < NSP; ++w)
+#pragma unroll
+        for (int m = 0; m < E; ++m) ex.template put<0, 0>(w, j0 + m * (N / E), F[w][m]);
+      ex.sync();
+#pragma unroll
+      for (int w = 0; w < NFW; ++w) {
+        const bool split = w < NSP;
+        V* ca = C + ((long long)(2 * w) * rows + rrow) * kxp;
+        V* cb = C + ((long long)(2 * w + 1) * rows + rrow) * kxp;
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+          const int k = j0 + m * (N / E);
+          if (rvalid && k < kend) {
+            V va = czero<V>(), vb = czero<V>();
+            if (k <= g.Kx) {
+              const V Fk = F[w][m];
+              if (split) {
+                const V Fm = cconj(ex.template get<0, 0>(w, k == 0 ? 0 : N - k));
+                va = cscale(cadd(Fk, Fm), T(0.5));
+                vb = cscale(cmul_mi(csub(Fk, Fm)), T(0.5));
+              } else {
+                va = Fk;
+              }
+            }
+            ca[k] = va;
+            if (split) cb[k] = vb;
+          }
         }
       }
     }
   }
+  }
 }
 
 template <typename T, int N, int NG, int NSC>
-__global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v),
-                                  NG == 1 && NSC == 0 ? MinB<T, N>::xpass : 1)
+__global__ void __launch_bounds__(RPCOf<T, N, NG == 1 && NSC == 0>::v * (N / EPass<T, N, 3>::v),
+                                  NG == 1 && NSC == 0 ? MinB<T, N>::xpass : MinB<T, N>::xmulti)
     k_xpass(const PassArgs a, const int rpc) {
   using V = typename cplx<T>::type;
   using FV = typename fft_of<V>::val;
@@ -656,8 +821,8 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v),
   const long long ngroups = (rows + rpc - 1) / rpc;
   V* stage = reinterpret_cast<V*>(smraw);
   V* exbuf = stage + NF * rpc * kxp;
-  // exchange region of this row: XLINES lines of N slots, single buffer
-  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLINES * N, N, 0, 0};
+  // exchange region of this row: XLines lines of N slots, single buffer
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLines<T, N, NG == 1 && NSC == 0>::v * N, N, 0, 0};
   // rows are independent between the group barriers: sync only the row's threads
   if (G >= 32) {
     ex.bar_id = 1 + rl;
@@ -675,7 +840,7 @@ __global__ void __launch_bounds__(RPCOf<T, N>::v * (N / EPass<T, N, 3>::v),
   if constexpr (TR) {
     tw.load(static_cast<const W*>(a.tw_x), j0);
   } else if constexpr (TT) {
-    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLINES * N);
+    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLines<T, N, NG == 1 && NSC == 0>::v * N);
     if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const W*>(a.tw_x), j0);
     tw = TwAcc{twt, j0};
   } else {
@@ -1104,13 +1269,13 @@ cudaError_t yinv_n(const PassArgs& a, cudaStream_t s) {
   PS_SHAPE_DISPATCH(yinv_nv, a.shape[1], a, s);
 }
 // Shared memory of the x pass for rpc rows: one input stage of 6 ng rows, the
-// exchange region (XLINES lines per row) and, when used, the twiddle table.
-template <typename T, int N>
+// exchange region (XLines lines per row) and, when used, the twiddle table.
+template <typename T, int N, bool HD = true>
 size_t xpass_smem(const Geo& g, int rpc, int nf) {
   using V = typename cplx<T>::type;
   constexpr int E = EPass<T, N, 3>::v;
   const size_t tt = (!XTwReg<T, N>::v && XTwTable<T, N>::v) ? (size_t)TwSlots<N, E>::total * (N / E) : 0;
-  return ((size_t)nf * rpc * g.kxp + (size_t)XLINES * rpc * N + tt) * sizeof(V);
+  return ((size_t)nf * rpc * g.kxp + (size_t)XLines<T, N, HD>::v * rpc * N + tt) * sizeof(V);
 }
 
 template <typename T, int N, int NG, int NSC>
@@ -1120,14 +1285,18 @@ cudaError_t xpass_ng(const PassArgs& a0, cudaStream_t s) {
   constexpr int NF = 6 * NG + 3 * NSC;
   constexpr int E = EPass<T, N, 3>::v, G = N / E;
   // rows per CTA: as many as the launch bound allows while two CTAs fit an SM
-  int rpc = RPCOf<T, N>::v;
-  while (rpc > 1 && xpass_smem<T, N>(a.g, rpc, NF) > 113 * 1024) rpc /= 2;
+  constexpr bool HD = NG == 1 && NSC == 0;
+  int rpc = RPCOf<T, N, HD>::v;
+  // (three where the launch bounds ask for three)
+  constexpr int per = XLines<T, N, HD>::v == 3 ? 2 : HD ? MinB<T, N>::xpass : MinB<T, N>::xmulti;
+  const size_t room = (per >= 5 ? 44 : per == 4 ? 56 : per == 3 ? 75 : 113) * 1024;
+  while (rpc > 1 && xpass_smem<T, N, HD>(a.g, rpc, NF) > room) rpc /= 2;
   const long long rows = (long long)a.g.nz * a.g.ny;
   // and fewer (down to a warp's worth) while that leaves SMs without two CTAs
   const long long beside = a.beside ? a.beside : 1;
   while (rpc > 1 && rpc * G > 32 && (rows + rpc - 1) / rpc * beside < 2 * NSM) rpc /= 2;
   if (a.xrpc > 0 && a.xrpc < rpc) rpc = a.xrpc;  // tuned (smaller) row groups
-  const size_t smem = xpass_smem<T, N>(a.g, rpc, NF);
+  const size_t smem = xpass_smem<T, N, HD>(a.g, rpc, NF);
   cudaError_t e = cudaFuncSetAttribute(k_xpass<T, N, NG, NSC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per_sm = 0;

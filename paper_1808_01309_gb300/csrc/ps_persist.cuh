@@ -97,7 +97,7 @@ __device__ __forceinline__ void ens_xpass_tile(const PassArgs& a, const int tile
   const int tid = threadIdx.x, j0 = tid % G, rl = tid / G;
   using FV = typename fft_of<V>::val;
   using W = typename fft_of<V>::tw;
-  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(smraw) + rl * XLINES * N, N, 0, 0};
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(smraw) + rl * XLines<T, N>::v * N, N, 0, 0};
   ex.bar_id = -1;
   const GlobalTw<W> tw{static_cast<const W*>(a.tw_x)};
   const long long rows = (long long)a.g.nz * a.g.ny;
@@ -246,7 +246,7 @@ EnsShape ens_shape_n(int kind, const Geo& g, int nfield) {
     const long long rows = (long long)g.nz * g.ny;
     s.ntiles = (int)((rows + RPC - 1) / RPC);
     s.gx = RPC;
-    s.smem = (size_t)XLINES * RPC * N * sizeof(V);
+    s.smem = (size_t)XLines<T, N>::v * RPC * N * sizeof(V);
   }
   return s;
 }
