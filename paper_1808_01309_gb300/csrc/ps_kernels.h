@@ -90,7 +90,7 @@ struct PassArgs {
   int* err;          // device error word (bounded waits that gave up), never null
   unsigned wait_polls;  // x pass: polls before a wait gives up (0 = PS_WAIT_LIMIT)
   int wait_test;     // x pass: test hook, the first copy of every CTA is never issued
-  const void* extra; // compact closure term added to the velocity group before projection, or null
+  const void* tau;   // compact model stress (six fields), whose -div joins the velocity group, or null
   // Constants in the working precision, set by prepare_args() on the host so
   // that FP32 kernels convert or divide no double on the GPU's slow FP64 pipe
   float dtf, nuf, etaf, nbvf, inv_n3f;
@@ -144,22 +144,29 @@ template <typename T>
 cudaError_t launch_diag_spectral(const Geo& g, Spec u, double* part, int nshells, int eq, cudaStream_t s);
 cudaError_t launch_diag_final(const double* part, int nblk, int nshells, double* out, cudaStream_t s);
 
-// LES closure (ps_les.cu): -i k_j tau_hat_ij of the model stress of the state
-// `in`, written to the compact buffer s.extra ([3][cz][cy][kxp], FP32).
+// LES closure (ps_les.cu).
 struct LesScratch {
   const float* params;  // MLP parameters (PS_MLP_NPARAM)
   const float* norm;    // mean[5], 1/std[5], s_tau, 1/s_A (device)
-  float2* spec;         // [9][nz][ny][nh]
+  // Buffers of the passes of a right-hand side with the closure (PassArgs::a6
+  // and b6): 15 z-inverse or y-inverse fields (u, omega, grad u) and 9 forward
+  // ones (n, tau).  spec ([9][nz][ny][nh] in training) is b15.
+  float2* a15;
+  float2* spec;
   float* phys;          // [9][nz][ny][nx]
   float* X;             // [P][5]
   float* Y;             // [P][6]
-  float2* extra;        // compact closure term
+  float2* extra;        // compact closure term (training)
   float* Arows;         // [P][9] gradient rows (training only)
 };
 cudaError_t launch_stream_copy(const void* src, void* dst, size_t bytes, int nsm, cudaStream_t s);
 cudaError_t launch_copy_cube(const void* src, void* dst, const Geo& g, int nc, size_t vb, int nsm, cudaStream_t s);
-cudaError_t les_closure_term(const Geo& g, Spec in, const void* twx, const void* twy, const void* twz,
-                             const LesScratch& s, cudaStream_t st);
+// The gradient of the stage input a.in through the backward z transform, into
+// fields 6..14 of a.a6.
+cudaError_t launch_les_grad_z(const PassArgs& a, cudaStream_t s);
+// Fields 6..14 of a.b6 to physical space, the network, and the model stress
+// through the forward x transform, into fields 3..8 of a.a6 (three kernels).
+cudaError_t launch_les_stress(const PassArgs& a, const LesScratch& sc, cudaStream_t s);
 // Force loss (sum over the half spectrum of w |D P(closure) - f|^2) of the
 // state `in` against the subgrid force f (full layout), added to *loss, and
 // its parameter gradient added to grad; params replaces s.params.

@@ -1,8 +1,13 @@
 // Learned LES closure on the CUDA path (include/ps.h: ps_plan_set_closure,
 // ps_les_training_sample): plain (unpruned) 3D transforms of any number of
 // fields, the resolved velocity-gradient invariants, the MLP of ps_mlp.cu, and
-// the divergence of the modelled stress that the z-forward pass adds to the
-// nonlinear term before the projection.  FP32.
+// the model stress.  FP32.
+//
+// In a step the closure shares the passes of the right-hand side: the nine
+// gradient fields ride behind u and omega through the y-inverse pass, the six
+// stress fields behind n through the y- and z-forward passes, all pruned to the
+// retained modes, and the update kernel adds the divergence of the stress to
+// the nonlinear term before the projection.
 #include <cmath>
 #include <string>
 #include <vector>
@@ -261,46 +266,49 @@ __global__ void k_grad(const Geo g, const Spec u, V* out) {
     for (int b = 0; b < 3; ++b) out[(3 * a + b) * total + i] = cmul_i(cscale(uu[a], k[b]));
 }
 
-// Invariants tr S^2, tr R^2, tr S^3, tr S R^2, tr S^2 R^2 of A (9 physical
-// fields), standardised: X[p][n] = (lambda_n - mean_n) * invstd_n, with
-// norm = [mean 5 | invstd 5 | s_tau | 1/s_A].  Aout (optional) receives the
-// gradient as rows [p][9].
-__global__ void k_features(const float* __restrict__ A, float* __restrict__ X, float* __restrict__ Aout,
-                           long long P, const float* __restrict__ norm) {
-  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  float a[3][3], S[3][3], R[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) a[i][j] = A[(3 * i + j) * P + p];
-  if (Aout) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Aout[p * 9 + k] = a[k / 3][k % 3];
-  }
+// Invariants tr S^2, tr R^2, tr S^3, tr S R^2, tr S^2 R^2 of the gradient a[3 i + j].
+__device__ __forceinline__ void invariants(const float (&a)[9], float (&lam)[5]) {
+  float S[3][3], R[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      S[i][j] = 0.5f * (a[i][j] + a[j][i]);
-      R[i][j] = 0.5f * (a[i][j] - a[j][i]);
+      S[i][j] = 0.5f * (a[3 * i + j] + a[3 * j + i]);
+      R[i][j] = 0.5f * (a[3 * i + j] - a[3 * j + i]);
     }
   float S2[3][3], R2[3][3];
   matmul3(S, S, S2);
   matmul3(R, R, R2);
-  float l1 = 0, l2 = 0, l3 = 0, l4 = 0, l5 = 0;
+#pragma unroll
+  for (int n = 0; n < 5; ++n) lam[n] = 0.f;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    l1 += S2[i][i];
-    l2 += R2[i][i];
+    lam[0] += S2[i][i];
+    lam[1] += R2[i][i];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      l3 += S2[i][k] * S[k][i];
-      l4 += S[i][k] * R2[k][i];
-      l5 += S2[i][k] * R2[k][i];
+      lam[2] += S2[i][k] * S[k][i];
+      lam[3] += S[i][k] * R2[k][i];
+      lam[4] += S2[i][k] * R2[k][i];
     }
   }
-  const float lam[5] = {l1, l2, l3, l4, l5};
+}
+
+// Invariants of A (9 physical fields), standardised: X[p][n] = (lambda_n -
+// mean_n) * invstd_n, with norm = [mean 5 | invstd 5 | s_tau | 1/s_A].  Aout
+// (optional) receives the gradient as rows [p][9].
+__global__ void k_features(const float* __restrict__ A, float* __restrict__ X, float* __restrict__ Aout,
+                           long long P, const float* __restrict__ norm) {
+  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (p >= P) return;
+  float a[9], lam[5];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a[k] = A[k * P + p];
+  if (Aout) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) Aout[p * 9 + k] = a[k];
+  }
+  invariants(a, lam);
 #pragma unroll
   for (int n = 0; n < 5; ++n) X[p * 5 + n] = (lam[n] - norm[n]) * norm[5 + n];
 }
@@ -511,34 +519,220 @@ __global__ void k_dg(const float* __restrict__ Arows, const float* __restrict__ 
 
 }  // namespace les
 
-cudaError_t les_closure_term(const Geo& g, Spec in, const void* twx, const void* twy, const void* twz,
-                             const LesScratch& s, cudaStream_t st) {
-  using namespace les;
-  const long long P = (long long)g.nx * g.ny * g.nz;
-  const long long M = (long long)g.nz * g.ny * g.nh;
-  const V *tx = static_cast<const V*>(twx), *ty = static_cast<const V*>(twy), *tz = static_cast<const V*>(twz);
-  k_grad<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, in, s.spec);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.spec, s.phys, tx, ty, tz, st);
-  if (e == cudaSuccess) {
-    k_features<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(s.phys, s.X, nullptr, P, s.norm);
-    e = cudaGetLastError();
+namespace les {
+
+// Field 3 i + j of the velocity gradient, i k_j u_i, through the backward z
+// transform: retained lines only, out [9][nz][cy][kxp].  One field and tile per
+// CTA (blockIdx.z = field).
+template <int N>
+__global__ void __launch_bounds__(ColShape<float, N, 0>::NTH) k_grad_z(const Geo g, const Spec u, V* __restrict__ out,
+                                                                       const V* __restrict__ tw) {
+  using SH = ColShape<float, N, 0>;
+  constexpr int E = SH::E, G = SH::G, TX = SH::TX, NB = SH::NB;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  const int line = threadIdx.x % TX, rest = threadIdx.x / TX, j0 = rest % G, bb = rest / G;
+  const int iy = blockIdx.y * NB + bb, kx = blockIdx.x * TX + line, f = blockIdx.z, c = f / 3, d = f % 3;
+  const bool ok = iy < g.cy;
+  const int q = iy <= g.Ky ? iy : iy - g.cy;
+  ColumnExchange<V, ilog2<Sched<N, E>::R0>::v, 1, TX> ex{reinterpret_cast<V*>(smraw) + bb * N * TX, 0, TX, line, 0};
+  const V* pu = static_cast<const V*>(u.p) + c * u.cs + (long long)rowof(q, u.ywrap) * u.ys + kx;
+  const float kf = d == 0 ? float(kx) * g.sxf : float(q) * g.syf;
+  V x[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int r = sidx(j0 + m * (N / E), N);
+    V v = czero<V>();
+    if (ok && kx < g.cx && kept(g, kx, q, r))
+      v = cmul_i(cscale(__ldg(pu + (long long)rowof(r, u.zwrap) * u.zs), d == 2 ? float(r) * g.szf : kf));
+    x[m] = v;
   }
-  if (e == cudaSuccess) {
-    const ps_status ms = ps_mlp_forward(s.params, s.X, s.Y, P, st);
-    if (ms != PS_OK) return cudaErrorLaunchFailure;
+  line_fft<N, E, +1>(x, j0, tw, ex);
+  if (!ok) return;
+  V* o = out + (long long)f * g.nz * g.cy * g.kxp + (long long)iy * g.kxp + kx;
+#pragma unroll
+  for (int m = 0; m < E; ++m) o[(long long)LinePos<float, N, E>::out(j0, m) * g.cy * g.kxp] = x[m];
+}
+
+// Rows of the nine gradient fields (in [9][rows][kxp], retained kx) to physical
+// space: A (planar, as k_stress_x reads it) and the standardised invariants X.
+template <int N>
+__global__ void __launch_bounds__(128) k_grad_x(const Geo g, const V* __restrict__ in, float* __restrict__ A,
+                                                float* __restrict__ X, const V* __restrict__ tw,
+                                                const float* __restrict__ norm) {
+  constexpr int E = EOf<float, N>::v, G = N / E, RPC = 128 / G;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  const int j0 = threadIdx.x % G, rl = threadIdx.x / G;
+  const long long rows = (long long)g.nz * g.ny, P = rows * N, row = (long long)blockIdx.x * RPC + rl;
+  const bool ok = row < rows;
+  LinesExchange<V, 1> ex{reinterpret_cast<V*>(smraw) + rl * 3 * N, N, 0, 0};
+  if (G >= 32) {
+    ex.bar_id = 1 + rl;
+    ex.nthr = G;
+  } else {
+    ex.bar_id = -1;
   }
-  if (e == cudaSuccess) {
-    k_stress<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(s.phys, s.Y, P, s.norm);
-    e = cudaGetLastError();
+  const GlobalTw<V> twa{tw};
+  float nm[10];
+#pragma unroll
+  for (int i = 0; i < 10; ++i) nm[i] = __ldg(norm + i);
+  const V* pr = in + (ok ? row : 0) * g.kxp;
+  auto gather = [&](V(&x)[E], int f) {  // fields f and f + 1 (8: alone) as one complex line
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int n = j0 + m * (N / E);
+      const bool hi = n > N / 2;
+      const int p = hi ? N - n : n;
+      V a = czero<V>(), b = czero<V>();
+      if (ok && p <= g.Kx) {
+        a = __ldg(pr + (long long)f * rows * g.kxp + p);
+        if (f < 8) b = __ldg(pr + (long long)(f + 1) * rows * g.kxp + p);
+      }
+      if (hi) {
+        a = cconj(a);
+        b = cconj(b);
+      }
+      x[m] = mk<V>(a.x - b.y, a.y + b.x);
+    }
+  };
+  V L[3][E], S[2][E];
+#pragma unroll
+  for (int l = 0; l < 3; ++l) gather(L[l], 2 * l);
+  gather(S[0], 6);
+  gather(S[1], 8);
+  line_fft_rows<N, E, +1>(L, j0, twa, ex);
+  line_fft_rows<N, E, +1>(S, j0, twa, ex);
+  if (!ok) return;
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const long long p = row * N + j0 + m * (N / E);
+    const float a[9] = {L[0][m].x, L[0][m].y, L[1][m].x, L[1][m].y, L[2][m].x, L[2][m].y, S[0][m].x, S[0][m].y, S[1][m].x};
+    float lam[5];
+    invariants(a, lam);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) A[k * P + p] = a[k];
+#pragma unroll
+    for (int n = 0; n < 5; ++n) X[p * 5 + n] = (lam[n] - nm[n]) * nm[5 + n];
   }
-  if (e == cudaSuccess) e = phys2spec(g, 6, s.phys, s.spec, tx, ty, tz, st);
-  if (e == cudaSuccess) {
-    const long long C = (long long)g.cz * g.cy * g.cx;
-    k_div<<<(unsigned)((C + 255) / 256), 256, 0, st>>>(g, s.spec, s.extra);
-    e = cudaGetLastError();
+}
+
+// The model stress tau = s_tau sum_n Y[p][n] T_n(A/s_A) of a row and its forward
+// x transform: six fields out [6][rows][kxp].
+template <int N>
+__global__ void __launch_bounds__(128) k_stress_x(const Geo g, const float* __restrict__ A, const float* __restrict__ Y,
+                                                  V* __restrict__ out, const V* __restrict__ tw,
+                                                  const float* __restrict__ norm) {
+  constexpr int E = EOf<float, N>::v, G = N / E, RPC = 128 / G;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  const int j0 = threadIdx.x % G, rl = threadIdx.x / G;
+  const long long rows = (long long)g.nz * g.ny, P = rows * N, row = (long long)blockIdx.x * RPC + rl;
+  const bool ok = row < rows;
+  LinesExchange<V, 1> ex{reinterpret_cast<V*>(smraw) + rl * 3 * N, N, 0, 0};
+  if (G >= 32) {
+    ex.bar_id = 1 + rl;
+    ex.nthr = G;
+  } else {
+    ex.bar_id = -1;
   }
-  return e;
+  const GlobalTw<V> twa{tw};
+  const float s_tau = __ldg(norm + 10), inv_sA = __ldg(norm + 11);
+  V F[3][E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const long long p = (ok ? row : 0) * N + j0 + m * (N / E);
+    float a[3][3], t[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) a[k / 3][k % 3] = __ldg(A + k * P + p);
+    float Tb[6][6];
+    tensor_basis(a, inv_sA, Tb);
+#pragma unroll
+    for (int n = 0; n < 6; ++n) {
+      const float y = __ldg(Y + p * 6 + n);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) t[k] += y * Tb[n][k];
+    }
+#pragma unroll
+    for (int w = 0; w < 3; ++w) F[w][m] = mk<V>(s_tau * t[2 * w], s_tau * t[2 * w + 1]);
+  }
+  line_fft_rows<N, E, -1>(F, j0, twa, ex);
+#pragma unroll
+  for (int w = 0; w < 3; ++w)
+#pragma unroll
+    for (int m = 0; m < E; ++m) ex.template put<0, 0>(w, j0 + m * (N / E), F[w][m]);
+  ex.sync();
+  const int kend = g.kxp < N / 2 + 1 ? g.kxp : N / 2 + 1;
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int k = j0 + m * (N / E);
+    if (ok && k < kend) {
+#pragma unroll
+      for (int w = 0; w < 3; ++w) {
+        const V Fm = cconj(ex.template get<0, 0>(w, k == 0 ? 0 : N - k));
+        const bool keep = k <= g.Kx;
+        out[(2 * w * rows + row) * g.kxp + k] = keep ? cscale(cadd(F[w][m], Fm), 0.5f) : czero<V>();
+        out[((2 * w + 1) * rows + row) * g.kxp + k] = keep ? cscale(cmul_mi(csub(F[w][m], Fm)), 0.5f) : czero<V>();
+      }
+    }
+  }
+}
+
+template <int N>
+cudaError_t grad_z_n(const Geo& g, const Spec& in, V* out, const V* tw, cudaStream_t s) {
+  using SH = ColShape<float, N, 0>;
+  const size_t smem = (size_t)SH::NB * N * SH::TX * sizeof(V);
+  const cudaError_t e = prep(k_grad_z<N>, smem);
+  if (e != cudaSuccess) return e;
+  k_grad_z<N><<<dim3(g.kxp / SH::TX, (g.cy + SH::NB - 1) / SH::NB, 9), SH::NTH, smem, s>>>(g, in, out, tw);
+  return cudaGetLastError();
+}
+template <int N>
+cudaError_t grad_x_n(const Geo& g, const V* in, float* A, float* X, const V* tw, const float* norm, cudaStream_t s) {
+  constexpr int G = N / EOf<float, N>::v, RPC = 128 / G;
+  const size_t smem = 3ull * RPC * N * sizeof(V);
+  const cudaError_t e = prep(k_grad_x<N>, smem);
+  if (e != cudaSuccess) return e;
+  const unsigned ctas = (unsigned)(((long long)g.nz * g.ny + RPC - 1) / RPC);
+  k_grad_x<N><<<ctas, RPC * G, smem, s>>>(g, in, A, X, tw, norm);
+  return cudaGetLastError();
+}
+template <int N>
+cudaError_t stress_x_n(const Geo& g, const float* A, const float* Y, V* out, const V* tw, const float* norm,
+                       cudaStream_t s) {
+  constexpr int G = N / EOf<float, N>::v, RPC = 128 / G;
+  const size_t smem = 3ull * RPC * N * sizeof(V);
+  const cudaError_t e = prep(k_stress_x<N>, smem);
+  if (e != cudaSuccess) return e;
+  const unsigned ctas = (unsigned)(((long long)g.nz * g.ny + RPC - 1) / RPC);
+  k_stress_x<N><<<ctas, RPC * G, smem, s>>>(g, A, Y, out, tw, norm);
+  return cudaGetLastError();
+}
+
+}  // namespace les
+
+cudaError_t launch_les_grad_z(const PassArgs& a, cudaStream_t s) {
+  les::V* out = static_cast<les::V*>(a.a6) + 6LL * a.g.nz * a.g.cy * a.g.kxp;
+#define CALL(N) les::grad_z_n<N>(a.g, a.in, out, static_cast<const les::V*>(a.tw_z), s)
+  LES_DISPATCH(a.g.nz, CALL)
+#undef CALL
+}
+
+cudaError_t launch_les_stress(const PassArgs& a, const LesScratch& sc, cudaStream_t s) {
+  const long long rows = (long long)a.g.nz * a.g.ny;
+  const les::V* in = static_cast<const les::V*>(a.b6) + 6 * rows * a.g.kxp;
+  les::V* out = static_cast<les::V*>(a.a6) + 3 * rows * a.g.kxp;
+  const les::V* tw = static_cast<const les::V*>(a.tw_x);
+  auto grad = [&] {
+#define CALL(N) les::grad_x_n<N>(a.g, in, sc.phys, sc.X, tw, sc.norm, s)
+    LES_DISPATCH(a.g.nx, CALL)
+#undef CALL
+  };
+  auto stress = [&] {
+#define CALL(N) les::stress_x_n<N>(a.g, sc.phys, sc.Y, out, tw, sc.norm, s)
+    LES_DISPATCH(a.g.nx, CALL)
+#undef CALL
+  };
+  cudaError_t e = grad();
+  if (e == cudaSuccess && ps_mlp_forward(sc.params, sc.X, sc.Y, rows * a.g.nx, s) != PS_OK) e = cudaErrorLaunchFailure;
+  return e == cudaSuccess ? stress() : e;
 }
 
 cudaError_t les_closure_grad(const Geo& g, Spec in, Spec f, const void* twx, const void* twy, const void* twz,

@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(ColShape<T, N, 2, VAR>::NTH, MinB<T, N>::zfwd)
 // retained set are written as zero); otherwise one thread per retained mode.
 // Consecutive threads take consecutive kx: every access is a contiguous row.
 // ---------------------------------------------------------------------------
-template <typename T, int NG, int NSC, bool SLAB, bool COH>
+template <typename T, int NG, int NSC, bool SLAB, bool COH, bool LES = false>
 __device__ __forceinline__ void update_mode(const PassArgs& a, const int full, const unsigned idx) {
   using V = typename cplx<T>::type;
   constexpr int NC = 3 * NG + NSC;  // state components
@@ -1074,11 +1074,13 @@ __device__ __forceinline__ void update_mode(const PassArgs& a, const int full, c
     } else {
       V v0 = ldv<COH>(nh + (c0 + 0) * ccs + ci), v1 = ldv<COH>(nh + (c0 + 1) * ccs + ci), v2 = ldv<COH>(nh + (c0 + 2) * ccs + ci);
       if (!mag) {
-        if (a.extra) {  // closure term (LES), compact layout
-          const V* ex0 = static_cast<const V*>(a.extra) + ci;
-          v0 = cadd(v0, ldv<COH>(ex0));
-          v1 = cadd(v1, ldv<COH>(ex0 + ccs));
-          v2 = cadd(v2, ldv<COH>(ex0 + 2 * ccs));
+        if constexpr (LES) {  // -i k_j tau_cj; components 11, 22, 33, 12, 13, 23
+          const V* t = static_cast<const V*>(a.tau) + ci;
+          const V t0 = ldv<COH>(t), t1 = ldv<COH>(t + ccs), t2 = ldv<COH>(t + 2 * ccs);
+          const V t3 = ldv<COH>(t + 3 * ccs), t4 = ldv<COH>(t + 4 * ccs), t5 = ldv<COH>(t + 5 * ccs);
+          v0 = cadd(v0, cmul_mi(cadd(cadd(cscale(t0, kxv), cscale(t3, kyv)), cscale(t4, kzv))));
+          v1 = cadd(v1, cmul_mi(cadd(cadd(cscale(t3, kxv), cscale(t1, kyv)), cscale(t5, kzv))));
+          v2 = cadd(v2, cmul_mi(cadd(cadd(cscale(t4, kxv), cscale(t5, kyv)), cscale(t2, kzv))));
         }
         const V* fb = static_cast<const V*>(a.fbox);
         if (fb && kx <= a.Fx && q <= a.Fy && q >= -a.Fy && r <= a.Fz && r >= -a.Fz) {
@@ -1176,9 +1178,9 @@ __device__ __forceinline__ void update_mode(const PassArgs& a, const int full, c
 
 // 32-bit mode index (the launcher checks that the modes fit): 64-bit integer
 // division runs on the FP64 pipe, which is slow on this GPU
-template <typename T, int NG, int NSC, bool SLAB = false>
+template <typename T, int NG, int NSC, bool SLAB = false, bool LES = false>
 __global__ void __launch_bounds__(256) k_update(const PassArgs a, const int full) {
-  update_mode<T, NG, NSC, SLAB, false>(a, full, blockIdx.x * blockDim.x + threadIdx.x);
+  update_mode<T, NG, NSC, SLAB, false, LES>(a, full, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1366,7 +1368,11 @@ cudaError_t update_launch(const PassArgs& a0, cudaStream_t s) {
   if (slab) k_update<T, 1, 0, true><<<blocks, 256, 0, s>>>(a, full);  // slabs: HD only
   else if (a.ng == 2) k_update<T, 2, 0><<<blocks, 256, 0, s>>>(a, full);
   else if (a.nsc) k_update<T, 1, 1><<<blocks, 256, 0, s>>>(a, full);
-  else k_update<T, 1, 0><<<blocks, 256, 0, s>>>(a, full);
+  else if (a.tau) {
+    if constexpr (sizeof(T) == 4) k_update<T, 1, 0, false, true><<<blocks, 256, 0, s>>>(a, full);
+    else return cudaErrorInvalidValue;  // the closure is FP32
+  } else
+    k_update<T, 1, 0><<<blocks, 256, 0, s>>>(a, full);
   return cudaGetLastError();
 }
 

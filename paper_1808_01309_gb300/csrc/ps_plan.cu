@@ -151,7 +151,7 @@ struct ps_plan {
   // learned LES closure (ps_plan_set_closure)
   bool les_on = false;
   ps::LesScratch les{};
-  void* les_mem[9] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  void* les_mem[10] = {};
   int ng = 1;    // 3-component groups: 1 HD and Boussinesq, 2 MHD
   Counts cn{1, 0, 3, 6, 3};
   Geo g{};
@@ -336,6 +336,7 @@ ps_status run_inverse_and_x(ps_plan* p, PassArgs& a) {
   int nb = 0;
   if ((s = launch(p, 0, [&] { return launch_zinv<T>(a, p->stream, &nb); }, "z-inverse pass")) != PS_OK) return s;
   p->n_epart_run = nb;
+  if (a.tau && (s = launch(p, 5, [&] { return launch_les_grad_z(a, p->stream); }, "LES gradient")) != PS_OK) return s;
   if ((s = launch(p, 1, [&] { return launch_yinv<T>(a, p->stream); }, "y-inverse pass")) != PS_OK) return s;
   if ((s = launch(p, 2, [&] { return launch_xpass<T>(a, p->stream); }, "x pass")) != PS_OK) return s;
   return PS_OK;
@@ -346,21 +347,25 @@ ps_status run_inverse_and_x(ps_plan* p, PassArgs& a) {
 template <typename T>
 ps_status run_rhs_passes(ps_plan* p, PassArgs& a) {
   ps_status s;
+  if (p->les_on) {
+    // the closure's fields ride behind the step's own (ps_les.cu)
+    a.a6 = p->les.a15;
+    a.b6 = p->les.spec;
+    a.nfi = 15;
+    a.nfo = 9;
+    a.tau = p->les.a15 + 3LL * p->g.cz * p->g.cy * p->g.kxp;
+  }
   if ((s = run_inverse_and_x<T>(p, a)) != PS_OK) return s;
   if (a.e_part) {
     if ((s = launch(p, 5, [&] { return launch_sum_partials(p->e_part, p->n_epart_run, p->stats, p->stream); },
                     "energy reduction")) != PS_OK)
       return s;
   }
-  if ((s = launch(p, 3, [&] { return launch_yfwd<T>(a, p->stream); }, "y-forward pass")) != PS_OK) return s;
-  if (p->les_on) {
-    // closure term of the stage input, added by the z-forward pass
-    if ((s = launch(p, 5, [&] { return les_closure_term(p->g, a.in, a.tw_x, a.tw_y, a.tw_z, p->les, p->stream); },
-                    "LES closure")) != PS_OK)
-      return s;
-    p->launches += 10;  // the closure is 11 kernels
-    a.extra = p->les.extra;
+  if (a.tau) {
+    if ((s = launch(p, 5, [&] { return launch_les_stress(a, p->les, p->stream); }, "LES stress")) != PS_OK) return s;
+    p->launches += 2;
   }
+  if ((s = launch(p, 3, [&] { return launch_yfwd<T>(a, p->stream); }, "y-forward pass")) != PS_OK) return s;
   if ((s = launch(p, 4, [&] { return launch_zfwd<T>(a, p->stream); }, "z-forward pass")) != PS_OK) return s;
   if ((s = launch(p, 6, [&] { return launch_update<T>(a, p->stream); }, "update")) != PS_OK) return s;
   return PS_OK;
@@ -515,7 +520,7 @@ void release(ps_plan* p) {
   void* bufs[] = {p->a6, p->b6, p->nxt, p->acc, p->tw, p->iftab, p->fbox, p->e_part, p->stats,
                   p->umax2, p->ext, p->err, p->dpart, p->dout, p->hstate, p->les_mem[0], p->les_mem[1],
                   p->les_mem[2], p->les_mem[3], p->les_mem[4], p->les_mem[5], p->les_mem[6], p->les_mem[7],
-                  p->les_mem[8]};
+                  p->les_mem[8], p->les_mem[9]};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (auto& t : p->tl) {
@@ -1097,10 +1102,13 @@ ps_status ps_plan_set_closure(ps_plan* p, const float* params, const double* nor
   const ps::Geo& g = p->g;
   const size_t P = (size_t)g.nx * g.ny * g.nz, M = (size_t)g.nz * g.ny * g.nh;
   if (!p->les_mem[0]) {
-    const size_t sizes[7] = {sizeof(float) * PS_MLP_NPARAM, sizeof(float) * 16, sizeof(float2) * 9 * M,
+    const size_t rows = (size_t)g.nz * g.ny * g.kxp, zrows = (size_t)g.nz * g.cy * g.kxp;
+    const size_t sizes[7] = {sizeof(float) * PS_MLP_NPARAM, sizeof(float) * 16,
+                             sizeof(float2) * std::max(9 * M, 15 * rows),
                              sizeof(float) * 9 * P, sizeof(float) * 5 * P, sizeof(float) * 6 * P,
                              sizeof(float2) * p->sz.cmp};
     for (int i = 0; i < 7; ++i) PS_CU(cudaMalloc(&p->les_mem[i], sizes[i]), "closure scratch");
+    PS_CU(cudaMalloc(&p->les_mem[9], sizeof(float2) * std::max(15 * zrows, 9 * rows)), "closure scratch");
     PS_CU(cudaMemsetAsync(p->les_mem[6], 0, sizes[6], p->stream), "closure scratch");
   }
   float h[12];
@@ -1121,6 +1129,7 @@ ps_status ps_plan_set_closure(ps_plan* p, const float* params, const double* nor
   p->les.X = static_cast<float*>(p->les_mem[4]);
   p->les.Y = static_cast<float*>(p->les_mem[5]);
   p->les.extra = static_cast<float2*>(p->les_mem[6]);
+  p->les.a15 = static_cast<float2*>(p->les_mem[9]);
   if (!p->les_on) drop_cached_graph(p);  // the closure launches join the step
   p->les_on = true;
   return PS_OK;
