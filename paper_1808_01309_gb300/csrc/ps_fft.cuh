@@ -188,13 +188,35 @@ __device__ __forceinline__ void dft3(V& a, V& b, V& c) {
   c = csub(t2, cmul_i(d));
 }
 
-// In-register DFT of size R in {2,3,4,6,8,16}.  R = 6 = 2 x 3: two 3-point
+// 12-point DFT as 3 x 4 without twiddles (Good's prime-factor map): the inputs
+// n = 4 n1 + 3 n2 (mod 12) through 4-point DFTs over n2 and 3-point DFTs over
+// n1, outputs k = 4 k1 + 9 k2 (mod 12).
+template <int DIR, typename V>
+__device__ __forceinline__ void dft12(V (&x)[12]) {
+  V y[3][4];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) y[i][j] = x[(4 * i + 3 * j) % 12];
+    dft_pow2<4, DIR>(y[i]);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    dft3<DIR>(y[0][j], y[1][j], y[2][j]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) x[(4 * i + 9 * j) % 12] = y[i][j];
+  }
+}
+
+// In-register DFT of size R in {2,3,4,6,8,12,16}.  R = 6 = 2 x 3: two 3-point
 // DFTs of the even and odd samples, then X[k] = A0[k] + w6^k A1[k] and
 // X[k+3] = A0[k] - w6^k A1[k], w6 = exp(DIR i pi/3).
 template <int R, int DIR, typename V>
 __device__ __forceinline__ void dft(V (&x)[R]) {
   if constexpr (R == 3) {
     dft3<DIR>(x[0], x[1], x[2]);
+  } else if constexpr (R == 12) {
+    dft12<DIR>(x);
   } else if constexpr (R == 6) {
     using T = decltype(V::x);
     constexpr double S3 = 0.86602540378443864676372317075293618347;
@@ -244,9 +266,9 @@ template <> struct Sched<512, 16> { static constexpr int S = 3, R0 = 16, R1 = 16
 template <> struct Sched<1024, 16> { static constexpr int S = 3, R0 = 16, R1 = 8, R2 = 8, R3 = 1; };
 template <> struct Sched<1024, 8> { static constexpr int S = 4, R0 = 8, R1 = 8, R2 = 8, R3 = 2; };
 // lengths with a factor 3 (E = 12)
-template <> struct Sched<48, 12> { static constexpr int S = 3, R0 = 6, R1 = 4, R2 = 2, R3 = 1; };
+template <> struct Sched<48, 12> { static constexpr int S = 2, R0 = 12, R1 = 4, R2 = 1, R3 = 1; };
 template <> struct Sched<96, 12> { static constexpr int S = 3, R0 = 6, R1 = 4, R2 = 4, R3 = 1; };
-template <> struct Sched<192, 12> { static constexpr int S = 4, R0 = 6, R1 = 4, R2 = 4, R3 = 2; };
+template <> struct Sched<192, 12> { static constexpr int S = 3, R0 = 12, R1 = 4, R2 = 4, R3 = 1; };
 
 // Registers per thread for a length-N line in precision T.
 template <typename T, int N> struct EOf {

@@ -78,18 +78,14 @@ template <typename T, int N> struct HasShapes {
   static constexpr bool v = sizeof(T) == 4 && (N == 64 || N == 96 || N == 128);
 };
 
-// x pass: lines per row transformed together (exchange region of a row).  The
-// FP32 hydrodynamic rows take three; the others one line at a time: with three,
-// registers and shared memory held the SM to eight warps (FP64), or six (MHD at
-// 256 points).
-#ifndef PS_XSEQ
-#define PS_XSEQ 0
-#endif
-#ifndef PS_XSEQB
-#define PS_XSEQB 3
-#endif
+// x pass: lines per row transformed together (exchange region of a row).  One at
+// a time leaves registers and shared memory for more rows per SM: with three an
+// SM held eight warps at FP64, six at MHD 256 points, eight at FP32 256 points
+// (131072 rows: 512 points 0.590 -> 0.553 ms; 65536 rows: 256 points 0.140 ->
+// 0.125, 128 points 0.081 -> 0.079).  FP32 rows of 12 points a thread
+// (multiples of three) gain nothing and keep three.
 template <typename T, int N, bool HD = true> struct XLines {
-  static constexpr int v = sizeof(T) == 4 && HD && !PS_XSEQ ? 3 : 1;
+  static constexpr int v = sizeof(T) == 4 && HD && N % 3 == 0 ? 3 : 1;
 };
 
 // rows per CTA in the x pass
@@ -124,9 +120,6 @@ template <typename T, int N> struct XTwReg {
 #endif
 #ifndef PS_MINB_XPASS
 #define PS_MINB_XPASS 2
-#endif
-#ifndef PS_MINB_X64
-#define PS_MINB_X64 3
 #endif
 #ifndef PS_MINB_Y1024
 #define PS_MINB_Y1024 2
@@ -180,7 +173,11 @@ template <typename T, int N> struct MinB {
   static constexpr int zinv = N == 1024 ? 1 : PS_MINB_ZINV;
   // x pass with two groups or a scalar: 96 to 192 registers hold the packed lines
   static constexpr int xmulti = sizeof(T) == 4 && EPass<T, N, 3>::v == 8 ? 3 : 2;
-  static constexpr int xpass = XLines<T, N>::v == 1 && sizeof(T) == 4 ? PS_XSEQB : sizeof(T) == 8 ? (N == 1024 || N % 3 == 0 ? 2 : PS_MINB_X64) : XHalved<T, N>::v ? 1 : PS_MINB_XPASS;
+  // (FP32 rows of 8 points a thread fit four CTAs of 128 threads at 128
+  // registers, those of 16 points three at 168)
+  static constexpr int xpass = XLines<T, N>::v == 3 ? (XHalved<T, N>::v ? 1 : PS_MINB_XPASS)
+                               : sizeof(T) == 8   ? (N == 1024 || N % 3 == 0 ? 2 : 3)
+                               : EPass<T, N, 3>::v == 8 ? 4 : 3;
   static constexpr int ypass = sizeof(T) == 4 && N == 1024 ? PS_MINB_Y1024 : sizeof(T) == 4 && N == 512 ? PS_MINB_Y512 : 0;
   static constexpr int zfwd = sizeof(T) == 4 && N == 1024 ? PS_MINB_ZF1024 : sizeof(T) == 4 && N == 512 ? PS_MINB_ZF512 : 0;
 };
@@ -1291,7 +1288,7 @@ cudaError_t xpass_ng(const PassArgs& a0, cudaStream_t s) {
   int rpc = RPCOf<T, N, HD>::v;
   // (three where the launch bounds ask for three)
   constexpr int per = XLines<T, N, HD>::v == 3 ? 2 : HD ? MinB<T, N>::xpass : MinB<T, N>::xmulti;
-  const size_t room = (per >= 5 ? 44 : per == 4 ? 56 : per == 3 ? 75 : 113) * 1024;
+  const size_t room = (per == 4 ? 56 : per == 3 ? 75 : 113) * 1024;
   while (rpc > 1 && xpass_smem<T, N, HD>(a.g, rpc, NF) > room) rpc /= 2;
   const long long rows = (long long)a.g.nz * a.g.ny;
   // and fewer (down to a warp's worth) while that leaves SMs without two CTAs
