@@ -12,13 +12,16 @@ cudaError_t launch_zinv<double>(const PassArgs& a, cudaStream_t s, int* nb) {
 
 template <int N>
 static int zinv_blocks_n(const Geo& g, int var) {
-  const int b0 = zinv_grid_blocks<double, N, 0>(g);
+  const int b0 = zinv_grid_blocks<double, N, 0>(g), b3 = zinv_grid_blocks<double, N, 3>(g);
+  int top = b0 > b3 ? b0 : b3;
   if constexpr (HasShapes<double, N>::v) {
     const int b1 = zinv_grid_blocks<double, N, 1>(g), b2 = zinv_grid_blocks<double, N, 2>(g);
-    if (var < 0) return b0 > b1 ? (b0 > b2 ? b0 : b2) : (b1 > b2 ? b1 : b2);
     if (var == 1) return b1;
     if (var == 2 && AltE<double, N>::v != EOf<double, N>::v) return b2;
+    top = top > b1 ? top : b1;
+    top = top > b2 ? top : b2;
   }
+  if (var < 0) return top;
   return b0;
 }
 

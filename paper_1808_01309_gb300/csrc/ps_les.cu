@@ -525,9 +525,9 @@ namespace les {
 // transform: retained lines only, out [9][nz][cy][kxp].  One field and tile per
 // CTA (blockIdx.z = field).
 template <int N>
-__global__ void __launch_bounds__(ColShape<float, N, 0>::NTH) k_grad_z(const Geo g, const Spec u, V* __restrict__ out,
+__global__ void __launch_bounds__(ColShape<float, N, 0, 3>::NTH) k_grad_z(const Geo g, const Spec u, V* __restrict__ out,
                                                                        const V* __restrict__ tw) {
-  using SH = ColShape<float, N, 0>;
+  using SH = ColShape<float, N, 0, 3>;
   constexpr int E = SH::E, G = SH::G, TX = SH::TX, NB = SH::NB;
   extern __shared__ __align__(128) unsigned char smraw[];
   const int line = threadIdx.x % TX, rest = threadIdx.x / TX, j0 = rest % G, bb = rest / G;
@@ -559,10 +559,10 @@ template <int N>
 __global__ void __launch_bounds__(128) k_grad_x(const Geo g, const V* __restrict__ in, float* __restrict__ A,
                                                 float* __restrict__ X, const V* __restrict__ tw,
                                                 const float* __restrict__ norm) {
-  constexpr int E = EOf<float, N>::v, G = N / E, RPC = 128 / G;
+  constexpr int E = EOf<float, N>::v, G = N / E;
   extern __shared__ __align__(128) unsigned char smraw[];
   const int j0 = threadIdx.x % G, rl = threadIdx.x / G;
-  const long long rows = (long long)g.nz * g.ny, P = rows * N, row = (long long)blockIdx.x * RPC + rl;
+  const long long rows = (long long)g.nz * g.ny, P = rows * N, row = (long long)blockIdx.x * (blockDim.x / G) + rl;
   const bool ok = row < rows;
   LinesExchange<V, 1> ex{reinterpret_cast<V*>(smraw) + rl * 3 * N, N, 0, 0};
   if (G >= 32) {
@@ -621,10 +621,10 @@ template <int N>
 __global__ void __launch_bounds__(128) k_stress_x(const Geo g, const float* __restrict__ A, const float* __restrict__ Y,
                                                   V* __restrict__ out, const V* __restrict__ tw,
                                                   const float* __restrict__ norm) {
-  constexpr int E = EOf<float, N>::v, G = N / E, RPC = 128 / G;
+  constexpr int E = EOf<float, N>::v, G = N / E;
   extern __shared__ __align__(128) unsigned char smraw[];
   const int j0 = threadIdx.x % G, rl = threadIdx.x / G;
-  const long long rows = (long long)g.nz * g.ny, P = rows * N, row = (long long)blockIdx.x * RPC + rl;
+  const long long rows = (long long)g.nz * g.ny, P = rows * N, row = (long long)blockIdx.x * (blockDim.x / G) + rl;
   const bool ok = row < rows;
   LinesExchange<V, 1> ex{reinterpret_cast<V*>(smraw) + rl * 3 * N, N, 0, 0};
   if (G >= 32) {
@@ -675,9 +675,17 @@ __global__ void __launch_bounds__(128) k_stress_x(const Geo g, const float* __re
   }
 }
 
+// Rows per CTA of the closure's x kernels: 128 threads, fewer (down to a warp)
+// while that leaves SMs without four CTAs.
+int row_group(long long rows, int G) {
+  int rpc = 128 / G;
+  while (rpc > 1 && rpc * G > 32 && (rows + rpc - 1) / rpc < 4 * NSM) rpc /= 2;
+  return rpc;
+}
+
 template <int N>
 cudaError_t grad_z_n(const Geo& g, const Spec& in, V* out, const V* tw, cudaStream_t s) {
-  using SH = ColShape<float, N, 0>;
+  using SH = ColShape<float, N, 0, 3>;
   const size_t smem = (size_t)SH::NB * N * SH::TX * sizeof(V);
   const cudaError_t e = prep(k_grad_z<N>, smem);
   if (e != cudaSuccess) return e;
@@ -686,23 +694,27 @@ cudaError_t grad_z_n(const Geo& g, const Spec& in, V* out, const V* tw, cudaStre
 }
 template <int N>
 cudaError_t grad_x_n(const Geo& g, const V* in, float* A, float* X, const V* tw, const float* norm, cudaStream_t s) {
-  constexpr int G = N / EOf<float, N>::v, RPC = 128 / G;
-  const size_t smem = 3ull * RPC * N * sizeof(V);
+  constexpr int G = N / EOf<float, N>::v;
+  const long long rows = (long long)g.nz * g.ny;
+  const int rpc = row_group(rows, G);
+  const size_t smem = 3ull * rpc * N * sizeof(V);
   const cudaError_t e = prep(k_grad_x<N>, smem);
   if (e != cudaSuccess) return e;
-  const unsigned ctas = (unsigned)(((long long)g.nz * g.ny + RPC - 1) / RPC);
-  k_grad_x<N><<<ctas, RPC * G, smem, s>>>(g, in, A, X, tw, norm);
+  const unsigned ctas = (unsigned)((rows + rpc - 1) / rpc);
+  k_grad_x<N><<<ctas, rpc * G, smem, s>>>(g, in, A, X, tw, norm);
   return cudaGetLastError();
 }
 template <int N>
 cudaError_t stress_x_n(const Geo& g, const float* A, const float* Y, V* out, const V* tw, const float* norm,
                        cudaStream_t s) {
-  constexpr int G = N / EOf<float, N>::v, RPC = 128 / G;
-  const size_t smem = 3ull * RPC * N * sizeof(V);
+  constexpr int G = N / EOf<float, N>::v;
+  const long long rows = (long long)g.nz * g.ny;
+  const int rpc = row_group(rows, G);
+  const size_t smem = 3ull * rpc * N * sizeof(V);
   const cudaError_t e = prep(k_stress_x<N>, smem);
   if (e != cudaSuccess) return e;
-  const unsigned ctas = (unsigned)(((long long)g.nz * g.ny + RPC - 1) / RPC);
-  k_stress_x<N><<<ctas, RPC * G, smem, s>>>(g, A, Y, out, tw, norm);
+  const unsigned ctas = (unsigned)((rows + rpc - 1) / rpc);
+  k_stress_x<N><<<ctas, rpc * G, smem, s>>>(g, A, Y, out, tw, norm);
   return cudaGetLastError();
 }
 

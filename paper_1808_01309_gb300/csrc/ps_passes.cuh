@@ -39,10 +39,11 @@ template <typename T, int K = 0> struct TXOf {
 };
 // Points per thread of pass K (0 z-inverse, 1 y passes, 2 z-forward, 3 x
 // pass).  At 1024 points FP32 every pass takes 16 (three stages, two
-// exchanges per line); the x pass then needs 231 registers and runs
-// without spills at one CTA per SM (MinB below): 10.98 ms per 1024^3 launch,
-// against 13.08 ms at 8 points per thread (four stages, three exchanges)
-// and 14.70 ms at 16 points capped to 128 registers (spills).
+// exchanges per line; 8 points: four stages, three exchanges).  512-point
+// column lines take 16 in pairs of threads (line_fft_paired; FP32 512^3
+// launches: y-inverse 0.753 -> 0.647 ms, y-forward 0.360 -> 0.311, z-forward
+// 0.298 -> 0.288), except in the z-inverse pass, whose input tile holds an SM
+// to two CTAs either way (0.658 ms at 8 points, 0.667 at 16).
 template <typename T, int N, int K> struct EPass {
   static constexpr int v = sizeof(T) == 4 && N == 512 && (K == 1 || K == 2) ? 16 : EOf<T, N>::v;
 };
@@ -58,7 +59,18 @@ template <typename T, int N, int K = 0> struct ColThreads {
 // Shape of column pass K (0 z-inverse, 1 y passes, 2 z-forward) on lines of
 // N points: kx columns per CTA (TX), points per thread (E), threads per line
 // (G), lines of the other index per CTA (NB, about 256 threads per CTA).
-// VAR 0 is the default above; VAR 1 halves the columns per CTA (twice the
+// VAR 0 (256 threads) is that of the ensemble's kernels and of plans whose
+// launches run beside others' (48 members: 12.5 ms for two steps, 13.1 with VAR
+// 3); VAR 3, the default of the per-pass launches, has the same columns and points
+// in smaller CTAs for lines of at most 256 points, whose barriers hold up fewer
+// warps and whose loads and transforms interleave: 64 threads up to 128 points,
+// else 128 (FP64 lengths with a factor 3: 128 measured better).  Launches of
+// FP32 z-inverse / y-inverse / z-forward passes, 256 threads -> VAR 3: 64 points
+// 28.8 / 24.7 / 12.3 -> 23.0 / 24.2 / 11.4 us, 96 points 24.7 / 23.1 / 10.4 ->
+// 20.6 / 20.7 / 10.4, 128 points 53.4 / 47.2 / 18.0 -> 50.1 / 43.1 / 16.5, 192
+// points 45.6 / 43.0 / 18.5 -> 39.1 / 39.0 / 16.5, 256 points 98 / 90 / 39 ->
+// 96 / 87 / 39; FP64 128 points 115 / 109 / 46 -> 93 / 96 / 41, 256 points 384 /
+// 432 / 176 -> 347 / 412 / 163 (y-forward 217 -> 226).  VAR 1 halves the columns per CTA (twice the
 // lines); VAR 2 takes the other radix schedule, 8 <-> 16 points per thread
 // (lengths with a factor 3 keep theirs).  Plans of the grids that the
 // ensemble tuner shapes (HasShapes) carry the variant per pass.
@@ -70,7 +82,8 @@ template <typename T, int N, int K, int VAR = 0> struct ColShape {
   static constexpr int TX = VAR == 1 ? TXOf<T, K>::v / 2 : TXOf<T, K>::v;
   static constexpr int E = VAR == 2 ? AltE<T, N>::v : EPass<T, N, K>::v;
   static constexpr int G = N / E;
-  static constexpr int q = 256 / (TX * G);
+  static constexpr int threads = VAR != 3 || N > 256 ? 256 : N > 128 || (sizeof(T) == 8 && N % 3 == 0) ? 128 : 64;
+  static constexpr int q = threads / (TX * G);
   static constexpr int NB = q < 1 ? 1 : q;
   static constexpr int NTH = TX * G * NB;
 };
@@ -84,14 +97,14 @@ template <typename T, int N> struct HasShapes {
 // (131072 rows: 512 points 0.590 -> 0.553 ms; 65536 rows: 256 points 0.140 ->
 // 0.125, 128 points 0.081 -> 0.079).  FP32 rows of 12 points a thread
 // (multiples of three) gain nothing and keep three.
-template <typename T, int N, bool HD = true> struct XLines {
-  static constexpr int v = sizeof(T) == 4 && HD && N % 3 == 0 ? 3 : 1;
+template <typename T, int N> struct XLines {
+  static constexpr int v = sizeof(T) == 4 && N % 3 == 0 ? 3 : 1;
 };
 
 // rows per CTA in the x pass
 template <typename T, int N, bool HD = true> struct RPCOf {
   static constexpr int G = N / EPass<T, N, 3>::v;
-  static constexpr int NT = XLines<T, N, HD>::v == 3 ? 256 : 128;  // threads per CTA
+  static constexpr int NT = XLines<T, N>::v == 3 && HD ? 256 : 128;  // threads per CTA
   static constexpr int v = G >= NT ? 1 : NT / G;
 };
 
@@ -129,9 +142,9 @@ template <typename T, int N> struct XTwReg {
 #endif
 // Exchange buffers of the y passes and the z-forward pass: one (two barriers
 // per exchange) for FP32 lines of 64 points and more, two (one barrier) else.
-// The single buffer lets more CTAs share an SM: four of 512 threads at 512
-// points (32 registers; 2 % faster than three CTAs with two buffers), two at
-// 1024 points (64 registers; two buffers of 128 KB held the SM to one CTA:
+// The single buffer lets more CTAs share an SM: four at 512 points (256
+// threads, 64 registers, one exchange per line: line_fft_paired), two at 1024
+// points (64 registers; two buffers of 128 KB held the SM to one CTA:
 // 1.3-1.4x slower), register-limited counts below (256^3 step 5 % faster).
 #ifndef PS_COLBUF512
 #define PS_COLBUF512 1
@@ -156,9 +169,8 @@ template <typename T, int N> struct ColBuf {
 // memory (stage + exchange above 113 KB at RPCOf rows; kx extent of the
 // 2/3 rule).  Its CTAs then have half the threads of the launch bound and
 // two of them fill the SM's shared memory, so the kernel may use the
-// registers of one full-size CTA per SM instead of spilling (FP32 256-point
-// rows: 0.152 -> 0.135 ms per 256^3 launch; 1024-point rows: 13.08 ->
-// 10.98 ms per 1024^3 launch).
+// registers of one full-size CTA per SM instead of spilling.  (Rows whose
+// lines are transformed three together only: FP32 multiples of three.)
 template <typename T, int N> struct XHalved {
   static constexpr long long kxp = ((N + 2) / 3 + 15) / 16 * 16;
   static constexpr int E = EPass<T, N, 3>::v, R = RPCOf<T, N>::v;
@@ -263,11 +275,9 @@ struct WorkTile {
 // One CTA tile (x, y) of the pass; gx = tiles along x (energy partial index
 // y gx + x).  COH: coherent loads (see ldv).
 //
-// SPLIT: the output fields of a tile are spread over blockIdx.z (zinv_slots):
-// one field per CTA, which stages only the components that field needs (with
-// energy partials the three velocity fields stay together, so the partials are
-// those of the whole tile).
-constexpr int zinv_slots(int ng, int nsc, bool epart) { return ng * (epart ? 4 : 6) + 3 * nsc; }
+// SPLIT: the output fields of a tile are spread over blockIdx.z, one per CTA,
+// which stages only the components that field needs and writes the energy
+// partial of its own component.
 template <typename T, int N, int NG, int NSC, bool COH, int VAR, bool SPLIT = false, class TL>
 __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   using V = typename cplx<T>::type;
@@ -300,14 +310,12 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   // gradient i k theta_hat is transformed (three fields)
   int g0 = 0, g1 = NG + NSC, f0 = 0, f1 = 0, c0 = 0, cstep = 1, nst = 0;
   if constexpr (SPLIT) {
-    const int per = a.e_part ? 4 : 6, slot = blockIdx.z;
-    g0 = slot < NG * per ? slot / per : NG;
+    g0 = blockIdx.z / 6;  // (the scalar's three fields come last)
     g1 = g0 + 1;
-    const int i = slot - g0 * per;  // field (or, with energy partials, the velocity triple first)
-    f0 = a.e_part && g0 < NG ? (i ? i + 2 : 0) : i;
-    f1 = a.e_part && g0 < NG && i == 0 ? 3 : f0 + 1;
-    // components: those of u, or the two of a curl component; theta
-    nst = g0 >= NG ? 1 : f0 >= 3 ? 2 : f1 - f0;
+    f0 = blockIdx.z - 6 * g0;
+    f1 = f0 + 1;
+    // components: that of u, or the two of a curl component; theta
+    nst = g0 < NG && f0 >= 3 ? 2 : 1;
     c0 = g0 >= NG ? 0 : f0 == 3 ? 1 : f0 > 3 ? 0 : f0;
     cstep = f0 == 4 ? 2 : 1;
   }
@@ -414,16 +422,17 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
   }
   __syncthreads();  // the tile is restaged for the next group
   }
-  if (SPLIT ? a.e_part && f0 == 0 : a.e_part != nullptr) {
+  if (SPLIT ? a.e_part && f0 < (g0 < NG ? 3 : 1) : a.e_part != nullptr) {
     // energy 1/2 sum w |u|^2 (+ |B|^2 or theta^2), w = 1 on the kx = 0 plane, else 2
     const double t = block_sum(esum * (kxg == 0 ? 0.5 : 1.0), red);
-    const int part = (SPLIT ? g0 * gridDim.y : 0) + tl.y();
+    const int part = (SPLIT ? (3 * g0 + f0) * gridDim.y : 0) + tl.y();
     if (threadIdx.x == 0) a.e_part[part * tl.gx() + tl.x()] = t;
   }
 }
 
 template <typename T, int N, int NG, int NSC, int VAR = 0, bool SPLIT = false>
-__global__ void __launch_bounds__(ColShape<T, N, 0, VAR>::NTH, MinB<T, N>::zinv) k_zinv(const PassArgs a) {
+__global__ void __launch_bounds__(ColShape<T, N, 0, VAR>::NTH,
+                                  VAR == 3 && N <= 256 ? 512 / ColShape<T, N, 0, VAR>::NTH : MinB<T, N>::zinv) k_zinv(const PassArgs a) {
   zinv_tile<T, N, NG, NSC, false, VAR, SPLIT>(a, LaunchTile{});
 }
 
@@ -476,8 +485,7 @@ __global__ void __launch_bounds__(ColShape<T, N, 1, VAR>::NTH, MinB<T, N>::ypass
 // the copies of the next group are issued into the same stage, so they land
 // while the current group is transformed.  Thread j0 of a row's group of G
 // threads holds the points n = j0 + m N/E.  The packed lines of a row are
-// transformed together (line_fft_rows): the inverse lines three at a time, the
-// forward lines of the products together, one exchange for all of them.
+// transformed one after the other, or three together (XLines).
 // NG = 2 (MHD): u + i omega and B + i j in, u x omega + j x B and u x B out.
 // NSC = 1 (Boussinesq): u + i omega and grad theta in, u x omega and
 // u . grad theta out.
@@ -639,9 +647,29 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
     }
   }
   gathered();
-  constexpr bool SEQ = XLines<T, N, HD>::v == 1;  // one line after the other
-  if constexpr (!SEQ) {
+  constexpr bool SEQ = XLines<T, N>::v == 1;  // one line after the other
+  if constexpr (!SEQ && HD) {
     rows_fft<N, E, +1>(U, j0, tw, ex);
+  } else if constexpr (!SEQ) {
+    // three lines together, then the other two or three
+    constexpr int R = NLI - 3;
+    V L[3][E], S[R][E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) L[c][m] = U[c][m];
+#pragma unroll
+      for (int c = 0; c < R; ++c) S[c][m] = U[3 + c][m];
+    }
+    rows_fft<N, E, +1>(L, j0, tw, ex);
+    rows_fft<N, E, +1>(S, j0, tw, ex);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) U[c][m] = L[c][m];
+#pragma unroll
+      for (int c = 0; c < R; ++c) U[3 + c][m] = S[c][m];
+    }
   } else {
     // one line after the other
 #pragma unroll
@@ -819,7 +847,7 @@ __global__ void __launch_bounds__(RPCOf<T, N, NG == 1 && NSC == 0>::v * (N / EPa
   V* stage = reinterpret_cast<V*>(smraw);
   V* exbuf = stage + NF * rpc * kxp;
   // exchange region of this row: XLines lines of N slots, single buffer
-  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLines<T, N, NG == 1 && NSC == 0>::v * N, N, 0, 0};
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLines<T, N>::v * N, N, 0, 0};
   // rows are independent between the group barriers: sync only the row's threads
   if (G >= 32) {
     ex.bar_id = 1 + rl;
@@ -837,7 +865,7 @@ __global__ void __launch_bounds__(RPCOf<T, N, NG == 1 && NSC == 0>::v * (N / EPa
   if constexpr (TR) {
     tw.load(static_cast<const W*>(a.tw_x), j0);
   } else if constexpr (TT) {
-    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLines<T, N, NG == 1 && NSC == 0>::v * N);
+    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLines<T, N>::v * N);
     if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const W*>(a.tw_x), j0);
     tw = TwAcc{twt, j0};
   } else {
@@ -1198,7 +1226,7 @@ int zinv_grid_blocks(const Geo& g) {
   return (g.kxp / SH::TX) * ((g.cy + SH::NB - 1) / SH::NB);
 }
 
-template <typename T, int N, int NG, int NSC, int VAR = 0>
+template <typename T, int N, int NG, int NSC, int VAR = 3>
 cudaError_t zinv_ng(const PassArgs& a0, cudaStream_t s, int* nb) {
   PassArgs a = a0;
   prepare_args(a);
@@ -1208,18 +1236,19 @@ cudaError_t zinv_ng(const PassArgs& a0, cudaStream_t s, int* nb) {
   const size_t smem = (1ull * NB * N * TX + 3ull * NB * a.g.cz * TX) * sizeof(V);
   dim3 grid(a.g.kxp / TX, (a.g.cy + NB - 1) / NB);
   if (nb) *nb = grid.x * grid.y;
-  // A grid of at most two CTAs per SM leaves SMs idle while each CTA transforms
-  // its six fields one after the other: spread the fields over CTAs instead
-  // (64^3 FP32 12.7 -> 5 us a launch).  Not where an ensemble's other members
-  // fill the SMs: there the components staged again cost more than they gain
-  // (48 members: 6.4 ms a step, 7.8 with both this and the smaller row groups).
-  if constexpr (VAR == 0) {
-    if ((long long)grid.x * grid.y * (a.beside ? a.beside : 1) <= 2 * NSM) {
-      cudaError_t e = prep(k_zinv<T, N, NG, NSC, 0, true>, smem);
+  // With CTAs (of 256 threads) for less than half the SMs the launch takes as long as one CTA's
+  // six transforms in a row: spread the fields over CTAs instead (64^3 FP32, 44
+  // CTAs: 12.7 -> 7.4 us).  Above that the components staged again cost more
+  // than they gain (128^3, 132 CTAs: a step 2 % slower; 256 CTAs: 15 to 20 %),
+  // as where an ensemble's other members fill the SMs (48 members: 6.4 ms a
+  // step, 7.8 with both this and the smaller row groups).
+  if constexpr (VAR == 3) {
+    if ((long long)grid.x * grid.y * (a.beside ? a.beside : 1) * SH::NTH <= NSM / 2 * 256) {
+      cudaError_t e = prep(k_zinv<T, N, NG, NSC, VAR, true>, smem);
       if (e != cudaSuccess) return e;
-      if (nb) *nb *= NG + NSC;
-      grid.z = zinv_slots(NG, NSC, a.e_part != nullptr);
-      k_zinv<T, N, NG, NSC, 0, true><<<grid, SH::NTH, smem, s>>>(a);
+      if (nb) *nb *= 3 * NG + NSC;
+      grid.z = 6 * NG + 3 * NSC;
+      k_zinv<T, N, NG, NSC, VAR, true><<<grid, SH::NTH, smem, s>>>(a);
       return cudaGetLastError();
     }
   }
@@ -1237,9 +1266,11 @@ cudaError_t zinv_n(const PassArgs& a, cudaStream_t s, int* nb) {
     if constexpr (AltE<T, N>::v != EOf<T, N>::v)
       if (a.shape[0] == 2) return zinv_ng<T, N, 1, 0, 2>(a, s, nb);
   }
+  if constexpr (N <= 256)
+    if (a.beside > 1) return zinv_ng<T, N, 1, 0, 0>(a, s, nb);
   return zinv_ng<T, N, 1, 0>(a, s, nb);
 }
-template <typename T, int N, int VAR = 0>
+template <typename T, int N, int VAR = 3>
 cudaError_t yinv_nv(const PassArgs& a0, cudaStream_t s) {
   PassArgs a = a0;
   prepare_args(a);
@@ -1261,7 +1292,9 @@ cudaError_t yinv_nv(const PassArgs& a0, cudaStream_t s) {
       if constexpr (AltE<T, N>::v != EOf<T, N>::v)                                      \
         if ((var_) == 2) return L<T, N, 2>(__VA_ARGS__);                                \
     }                                                                                   \
-    return L<T, N, 0>(__VA_ARGS__);                                                     \
+    if constexpr (N <= 256)                                                             \
+      if (a.beside > 1) return L<T, N, 0>(__VA_ARGS__);                                 \
+    return L<T, N, 3>(__VA_ARGS__);                                                     \
   } while (0)
 template <typename T, int N>
 cudaError_t yinv_n(const PassArgs& a, cudaStream_t s) {
@@ -1269,12 +1302,12 @@ cudaError_t yinv_n(const PassArgs& a, cudaStream_t s) {
 }
 // Shared memory of the x pass for rpc rows: one input stage of 6 ng rows, the
 // exchange region (XLines lines per row) and, when used, the twiddle table.
-template <typename T, int N, bool HD = true>
+template <typename T, int N>
 size_t xpass_smem(const Geo& g, int rpc, int nf) {
   using V = typename cplx<T>::type;
   constexpr int E = EPass<T, N, 3>::v;
   const size_t tt = (!XTwReg<T, N>::v && XTwTable<T, N>::v) ? (size_t)TwSlots<N, E>::total * (N / E) : 0;
-  return ((size_t)nf * rpc * g.kxp + (size_t)XLines<T, N, HD>::v * rpc * N + tt) * sizeof(V);
+  return ((size_t)nf * rpc * g.kxp + (size_t)XLines<T, N>::v * rpc * N + tt) * sizeof(V);
 }
 
 template <typename T, int N, int NG, int NSC>
@@ -1287,15 +1320,15 @@ cudaError_t xpass_ng(const PassArgs& a0, cudaStream_t s) {
   constexpr bool HD = NG == 1 && NSC == 0;
   int rpc = RPCOf<T, N, HD>::v;
   // (three where the launch bounds ask for three)
-  constexpr int per = XLines<T, N, HD>::v == 3 ? 2 : HD ? MinB<T, N>::xpass : MinB<T, N>::xmulti;
+  constexpr int per = XLines<T, N>::v == 3 ? 2 : HD ? MinB<T, N>::xpass : MinB<T, N>::xmulti;
   const size_t room = (per == 4 ? 56 : per == 3 ? 75 : 113) * 1024;
-  while (rpc > 1 && xpass_smem<T, N, HD>(a.g, rpc, NF) > room) rpc /= 2;
+  while (rpc > 1 && xpass_smem<T, N>(a.g, rpc, NF) > room) rpc /= 2;
   const long long rows = (long long)a.g.nz * a.g.ny;
-  // and fewer (down to a warp's worth) while that leaves SMs without two CTAs
+  // and fewer (down to a warp's worth) while that leaves SMs without a CTA
   const long long beside = a.beside ? a.beside : 1;
-  while (rpc > 1 && rpc * G > 32 && (rows + rpc - 1) / rpc * beside < 2 * NSM) rpc /= 2;
+  while (rpc > 1 && rpc * G > 32 && (rows + rpc - 1) / rpc * beside < NSM) rpc /= 2;
   if (a.xrpc > 0 && a.xrpc < rpc) rpc = a.xrpc;  // tuned (smaller) row groups
-  const size_t smem = xpass_smem<T, N, HD>(a.g, rpc, NF);
+  const size_t smem = xpass_smem<T, N>(a.g, rpc, NF);
   cudaError_t e = cudaFuncSetAttribute(k_xpass<T, N, NG, NSC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per_sm = 0;
@@ -1317,7 +1350,7 @@ cudaError_t xpass_n(const PassArgs& a, cudaStream_t s) {
   return a.nsc ? xpass_ng<T, N, 1, 1>(a, s) : xpass_ng<T, N, 1, 0>(a, s);
 }
 
-template <typename T, int N, int VAR = 0>
+template <typename T, int N, int VAR = 3>
 cudaError_t yfwd_nv(const PassArgs& a0, cudaStream_t s) {
   PassArgs a = a0;
   prepare_args(a);
@@ -1335,7 +1368,7 @@ template <typename T, int N>
 cudaError_t yfwd_n(const PassArgs& a, cudaStream_t s) {
   PS_SHAPE_DISPATCH(yfwd_nv, a.shape[1], a, s);
 }
-template <typename T, int N, int VAR = 0>
+template <typename T, int N, int VAR = 3>
 cudaError_t zfwd_nv(const PassArgs& a0, cudaStream_t s) {
   PassArgs a = a0;
   prepare_args(a);

@@ -679,8 +679,8 @@ ps_status ps_plan_create(const ps_config* cfg, void* cuda_stream, ps_plan** out)
   p->n_epart_run = p->n_epart;
   // room for the partials of every shape variant of the z-inverse pass
   const int nb = f32 ? zinv_blocks<float>(p->g, -1) : zinv_blocks<double>(p->g, -1);
-  // (one set per field group when the pass spreads the groups over CTAs)
-  ALLOC(p->e_part, sizeof(double) * (size_t)(nb > 0 ? nb : 1) * (p->ng + p->cn.nsc), "energy partials");
+  // (one set per component when the pass spreads the fields over CTAs)
+  ALLOC(p->e_part, sizeof(double) * (size_t)(nb > 0 ? nb : 1) * (3 * p->ng + p->cn.nsc), "energy partials");
   ALLOC(p->stats, sizeof(double) * 4, "stats");
   ALLOC(p->umax2, sizeof(unsigned long long), "max|u|");
   ALLOC(p->ext, sizeof(int) * 4, "forcing extent");
