@@ -433,6 +433,9 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
 template <typename T, int N, int NG, int NSC, int VAR = 0, bool SPLIT = false>
 __global__ void __launch_bounds__(ColShape<T, N, 0, VAR>::NTH,
                                   VAR == 3 && N <= 256 ? 512 / ColShape<T, N, 0, VAR>::NTH : MinB<T, N>::zinv) k_zinv(const PassArgs a) {
+  // the x pass of this right-hand side takes the maximum from zero (a memset
+  // before the step otherwise)
+  if (a.umax2 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.umax2 = 0ull;
   zinv_tile<T, N, NG, NSC, false, VAR, SPLIT>(a, LaunchTile{});
 }
 

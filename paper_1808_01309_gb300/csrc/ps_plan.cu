@@ -413,7 +413,6 @@ ps_status do_rk_step(ps_plan* p, void* uhat, double dt) {
     }
     p->if_dt = dt;
   }
-  PS_CU(cudaMemsetAsync(p->umax2, 0, sizeof(unsigned long long), p->stream), "reset max|u|");
   const int nst = p->cfg.rk_order == 4 ? 4 : 2;
   for (int st = 0; st < nst; ++st) {
     PassArgs a = stage_args(p, uhat, dt, st, true);
@@ -427,7 +426,6 @@ ps_status do_diag(ps_plan* p, const void* uhat, double* host_out) {
   ps_status s;
   const int w = DIAG_HEAD + p->nshells;
   PS_CU(cudaMemsetAsync(p->dpart, 0, sizeof(double) * (size_t)p->g.cz * w, p->stream), "diag reset");
-  PS_CU(cudaMemsetAsync(p->umax2, 0, sizeof(unsigned long long), p->stream), "diag reset");
   const Spec u = caller_spec(p->g, uhat);
   if ((s = launch(p, 5, [&] { return launch_diag_spectral<T>(p->g, u, p->dpart, p->nshells, (int)p->cfg.eq, p->stream); },
                   "spectral diagnostics")) != PS_OK)
