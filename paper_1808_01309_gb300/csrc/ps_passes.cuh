@@ -96,9 +96,11 @@ template <typename T, int N> struct HasShapes {
 // SM held eight warps at FP64, six at MHD 256 points, eight at FP32 256 points
 // (131072 rows: 512 points 0.590 -> 0.553 ms; 65536 rows: 256 points 0.140 ->
 // 0.125, 128 points 0.081 -> 0.079).  FP32 rows of 12 points a thread
-// (multiples of three) gain nothing and keep three.
-template <typename T, int N> struct XLines {
-  static constexpr int v = sizeof(T) == 4 && N % 3 == 0 ? 3 : 1;
+// (multiples of three) gain nothing and keep three, and so do those of 1024
+// points but for MHD (32768 rows: HD 0.351 ms with three, 0.358 with one; MHD
+// 1.00 and 0.76).
+template <typename T, int N, bool MHD = false> struct XLines {
+  static constexpr int v = sizeof(T) == 4 && (N % 3 == 0 || (N == 1024 && !MHD)) ? 3 : 1;
 };
 
 // rows per CTA in the x pass
@@ -650,7 +652,7 @@ __device__ __forceinline__ void xpass_row(const PassArgs& a, const long long row
     }
   }
   gathered();
-  constexpr bool SEQ = XLines<T, N>::v == 1;  // one line after the other
+  constexpr bool SEQ = XLines<T, N, NG == 2>::v == 1;  // one line after the other
   if constexpr (!SEQ && HD) {
     rows_fft<N, E, +1>(U, j0, tw, ex);
   } else if constexpr (!SEQ) {
@@ -850,7 +852,7 @@ __global__ void __launch_bounds__(RPCOf<T, N, NG == 1 && NSC == 0>::v * (N / EPa
   V* stage = reinterpret_cast<V*>(smraw);
   V* exbuf = stage + NF * rpc * kxp;
   // exchange region of this row: XLines lines of N slots, single buffer
-  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLines<T, N>::v * N, N, 0, 0};
+  LinesExchange<FV, 1> ex{reinterpret_cast<FV*>(exbuf) + rl * XLines<T, N, NG == 2>::v * N, N, 0, 0};
   // rows are independent between the group barriers: sync only the row's threads
   if (G >= 32) {
     ex.bar_id = 1 + rl;
@@ -868,7 +870,7 @@ __global__ void __launch_bounds__(RPCOf<T, N, NG == 1 && NSC == 0>::v * (N / EPa
   if constexpr (TR) {
     tw.load(static_cast<const W*>(a.tw_x), j0);
   } else if constexpr (TT) {
-    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLines<T, N>::v * N);
+    W* twt = reinterpret_cast<W*>(exbuf + rpc * XLines<T, N, NG == 2>::v * N);
     if (rl == 0) fill_thread_tw<N, E>(twt, static_cast<const W*>(a.tw_x), j0);
     tw = TwAcc{twt, j0};
   } else {
@@ -1305,12 +1307,12 @@ cudaError_t yinv_n(const PassArgs& a, cudaStream_t s) {
 }
 // Shared memory of the x pass for rpc rows: one input stage of 6 ng rows, the
 // exchange region (XLines lines per row) and, when used, the twiddle table.
-template <typename T, int N>
+template <typename T, int N, bool MHD = false>
 size_t xpass_smem(const Geo& g, int rpc, int nf) {
   using V = typename cplx<T>::type;
   constexpr int E = EPass<T, N, 3>::v;
   const size_t tt = (!XTwReg<T, N>::v && XTwTable<T, N>::v) ? (size_t)TwSlots<N, E>::total * (N / E) : 0;
-  return ((size_t)nf * rpc * g.kxp + (size_t)XLines<T, N>::v * rpc * N + tt) * sizeof(V);
+  return ((size_t)nf * rpc * g.kxp + (size_t)XLines<T, N, MHD>::v * rpc * N + tt) * sizeof(V);
 }
 
 template <typename T, int N, int NG, int NSC>
@@ -1323,15 +1325,15 @@ cudaError_t xpass_ng(const PassArgs& a0, cudaStream_t s) {
   constexpr bool HD = NG == 1 && NSC == 0;
   int rpc = RPCOf<T, N, HD>::v;
   // (three where the launch bounds ask for three)
-  constexpr int per = XLines<T, N>::v == 3 ? 2 : HD ? MinB<T, N>::xpass : MinB<T, N>::xmulti;
+  constexpr int per = XLines<T, N, NG == 2>::v == 3 ? 2 : HD ? MinB<T, N>::xpass : MinB<T, N>::xmulti;
   const size_t room = (per == 4 ? 56 : per == 3 ? 75 : 113) * 1024;
-  while (rpc > 1 && xpass_smem<T, N>(a.g, rpc, NF) > room) rpc /= 2;
+  while (rpc > 1 && xpass_smem<T, N, NG == 2>(a.g, rpc, NF) > room) rpc /= 2;
   const long long rows = (long long)a.g.nz * a.g.ny;
   // and fewer (down to a warp's worth) while that leaves SMs without a CTA
   const long long beside = a.beside ? a.beside : 1;
   while (rpc > 1 && rpc * G > 32 && (rows + rpc - 1) / rpc * beside < NSM) rpc /= 2;
   if (a.xrpc > 0 && a.xrpc < rpc) rpc = a.xrpc;  // tuned (smaller) row groups
-  const size_t smem = xpass_smem<T, N>(a.g, rpc, NF);
+  const size_t smem = xpass_smem<T, N, NG == 2>(a.g, rpc, NF);
   cudaError_t e = cudaFuncSetAttribute(k_xpass<T, N, NG, NSC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per_sm = 0;
