@@ -9,6 +9,7 @@
 // retained modes, and the update kernel adds the divergence of the stress to
 // the nonlinear term before the projection.
 #include <cmath>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -985,6 +986,53 @@ __global__ void k_truncate(const V* __restrict__ src, const Geo gs, V* __restric
   dst[i] = v;
 }
 
+// Scratch of ps_les_training_sample.  Mapping and unmapping its 0.3 GB took 0.3
+// of a call's 0.79 ms (256^3 to 64^3), and a training run calls it once per
+// snapshot: one block of at most SCRATCH_KEEP bytes is kept between calls.  A
+// call owns the block it takes (concurrent calls allocate their own) and has
+// synchronised its stream when it returns it; it is given back when a plan is
+// destroyed or an allocation here fails (scratch_trim).
+constexpr size_t SCRATCH_KEEP = 512ull << 20;
+struct Scratch {
+  void* p = nullptr;
+  size_t bytes = 0;
+  int device = -1;
+};
+std::mutex scratch_mutex;
+Scratch scratch_kept;
+
+Scratch scratch_kept_out() {
+  std::lock_guard<std::mutex> lock(scratch_mutex);
+  const Scratch s = scratch_kept;
+  scratch_kept = Scratch{};
+  return s;
+}
+cudaError_t scratch_take(size_t bytes, Scratch* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const Scratch k = scratch_kept_out();
+  if (k.p && k.device == dev && k.bytes >= bytes) {
+    *out = k;
+    return cudaSuccess;
+  }
+  cudaFree(k.p);
+  out->bytes = bytes;
+  out->device = dev;
+  return cudaMalloc(&out->p, bytes);
+}
+// ok: nothing the call launched is still running or has failed.
+void scratch_return(const Scratch& s, bool ok) {
+  if (ok && s.bytes <= SCRATCH_KEEP) {
+    std::lock_guard<std::mutex> lock(scratch_mutex);
+    if (!scratch_kept.p) {
+      scratch_kept = s;
+      return;
+    }
+  }
+  cudaFree(s.p);
+}
+
 Geo cube_geo(int n) {
   Geo g{};
   g.nx = g.ny = g.nz = n;
@@ -1001,6 +1049,9 @@ Geo cube_geo(int n) {
 unsigned blocks(long long n) { return (unsigned)((n + 255) / 256); }
 
 }  // namespace les
+
+void scratch_trim() { cudaFree(les::scratch_kept_out().p); }
+
 }  // namespace ps
 
 extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int n_les, int kc, const double* norm12,
@@ -1024,7 +1075,7 @@ extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int
   const Geo gd = cube_geo(n_dns), gl = cube_geo(n_les);
   const long long Md = (long long)gd.nz * gd.ny * gd.nh;
   const long long Ml = (long long)gl.nz * gl.ny * gl.nh, Pl = (long long)n_les * n_les * n_les;
-  // one allocation, cut into the transforms' buffers
+  // one block, cut into the transforms' buffers
   const long long cw = kc + 1, c2 = 2 * kc + 1;
   size_t need = 0;
   auto take = [&](size_t bytes) {
@@ -1041,13 +1092,14 @@ extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int
   const size_t o_sg = take(sizeof(V) * 9 * Ml);                   // transform scratch (9 fields)
   const size_t o_pl = take(sizeof(float) * 9 * Pl);               // LES physical (9 fields)
   const size_t o_nrm = take(sizeof(float) * 12);
-  char* base = nullptr;
+  Scratch scratch;
   ps_status st = PS_OK;
-  if (cudaMalloc(&base, need) != cudaSuccess) {
+  if (scratch_take(need, &scratch) != cudaSuccess) {
     (void)cudaGetLastError();
     set_last_error("ps_les_training_sample: device allocation failed");
     return PS_ERR_OOM;
   }
+  char* base = static_cast<char*>(scratch.p);
   auto cplx_at = [&](size_t o) { return reinterpret_cast<V*>(base + o); };
   V *twd = cplx_at(o_twd), *twl = cplx_at(o_twl), *sd = cplx_at(o_sd), *xb = cplx_at(o_xb), *yb = cplx_at(o_yb);
   V *ub = cplx_at(o_ub), *sl = cplx_at(o_sl), *sg = cplx_at(o_sg);
@@ -1110,8 +1162,8 @@ extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int
     set_last_error(std::string("ps_les_training_sample: ") + cudaGetErrorString(e));
     st = PS_ERR_CUDA;
   }
-  cudaStreamSynchronize(s);
-  cudaFree(base);
+  const cudaError_t es = cudaStreamSynchronize(s);
+  scratch_return(scratch, e == cudaSuccess && es == cudaSuccess);
   return st;
 }
 

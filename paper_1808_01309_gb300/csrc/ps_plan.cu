@@ -137,6 +137,8 @@ struct TimedLaunch {
 namespace ps {
 // Lets other translation units of the library report through ps_last_error().
 void set_last_error(const std::string& msg) { g_last_error = msg; }
+// Gives back the scratch block kept by ps_les_training_sample (ps_les.cu).
+void scratch_trim();
 }  // namespace ps
 
 struct ps_plan {
@@ -533,6 +535,7 @@ void release(ps_plan* p) {
   if (p->side_go) cudaEventDestroy(p->side_go);
   if (p->side_done) cudaEventDestroy(p->side_done);
   if (p->side) cudaStreamDestroy(p->side);
+  ps::scratch_trim();
 }
 
 }  // namespace
@@ -664,6 +667,11 @@ ps_status ps_plan_create(const ps_config* cfg, void* cuda_stream, ps_plan** out)
 #define ALLOC(ptr, bytes, what)                          \
   do {                                                   \
     cudaError_t e_ = cudaMalloc((void**)&(ptr), (bytes)); \
+    if (e_ == cudaErrorMemoryAllocation) {               \
+      (void)cudaGetLastError();                          \
+      ps::scratch_trim();                                \
+      e_ = cudaMalloc((void**)&(ptr), (bytes));          \
+    }                                                    \
     if (e_ != cudaSuccess) return bail(cuda_fail(e_, what)); \
   } while (0)
   ALLOC(p->a6, p->sz.a6 * vb, "scratch a");
