@@ -444,8 +444,10 @@ ps_status ps_plan_closure_grad_transfer(ps_plan* plan, const float* params, cons
  *             33, 12, 13, 23 (the part of the filtered momentum flux that an
  *             LES truncated at kc does not form itself)
  * n_dns, n_les in {16, 32, 48, 64, 96, 128, 192, 256, 512}, n_les <= n_dns,
- * 1 <= kc <= ceil(n_les/3) - 1.  Allocates and frees its scratch (about 60
- * bytes per DNS point); synchronises the stream. */
+ * 1 <= kc <= ceil(n_les/3) - 1.  Its scratch takes about 20 bytes per DNS
+ * point; a block of at most 512 MiB stays with the library between calls and
+ * is given back when a plan is destroyed or an allocation fails.  Synchronises
+ * the stream. */
 ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int n_les, int kc, const double* norm12, float* X,
                                  float* A, float* T, void* cuda_stream);
 
