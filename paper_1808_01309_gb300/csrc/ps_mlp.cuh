@@ -86,34 +86,28 @@ __device__ __forceinline__ void gelu_with_grad(float x, float& h, float& g) {
   g = 0.5f * (1.f + t) + 0.5f * x * (1.f - t * t) * C * (1.f + 3.f * 0.044715f * x * x);
 }
 
-// GELU (tanh form) of four values: 0.5 z (1 + tanh u) = z s with
-// s = 1/(1 + exp(-2u)), u = sqrt(2/pi) (z + 0.044715 z^3), for inference.  The
-// sigmoid takes one ex2 each and the four reciprocals come from one rcp of the
-// product, each refined by one Newton step; the rest runs two values per
-// instruction, since issue bounds the kernel (ten 64^3 closure steps 2905 ->
-// 2818 us against scalar operations with a compare and a select).  z is clamped
-// at -5.5 so that the product of four stays finite: there and below the result
-// is -5.9e-9 (1 + tanhf: up to 7.7e-8 off by cancellation).
+// GELU (tanh form) of four values, two of one sample (z[0], z[1]) and two of
+// another, for inference: 0.5 z (1 + tanh u) = z s with s = 1/(1 + exp(-2u)),
+// u = sqrt(2/pi) (z + 0.044715 z^3).  The sigmoid takes one ex2 each; the two
+// values of a sample share one rcp of their product, each refined by one Newton
+// step, and the rest runs two values per instruction, since issue bounds the
+// kernel.  A NaN thus stays within its own sample (one rcp for all four values
+// took it to the other one, and ten 64^3 closure steps 2744 instead of 2721 us).
+// z is clamped at -7.5 so that the product of two
+// and its reciprocal stay normal numbers: there and below the result is
+// -4.0e-18 (1 + tanhf: up to 7.7e-8 off by cancellation).
 __device__ __forceinline__ void gelu4(const float (&z)[4], float (&h)[4]) {
   constexpr float A = -2.f * 0.7978845608028654f * 1.4426950408889634f;  // -2 sqrt(2/pi) log2(e)
   constexpr float B = A * 0.044715f;
-  float2 x[2], s[2];
-  float d[4];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    x[i] = make_float2(clamp_low(z[2 * i], -5.5f), clamp_low(z[2 * i + 1], -5.5f));
-    const float2 v = mul2(x[i], fma2(mul2(x[i], x[i]), both(B), both(A)));
-    d[2 * i] = 1.f + ex2(v.x);
-    d[2 * i + 1] = 1.f + ex2(v.y);
-  }
-  const float p01 = d[0] * d[1], p23 = d[2] * d[3], r = rcp(p01 * p23);
-  const float r01 = r * p23, r23 = r * p01;
-  s[0] = make_float2(r01 * d[1], r01 * d[0]);
-  s[1] = make_float2(r23 * d[3], r23 * d[2]);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    s[i] = fma2(s[i], fma2(make_float2(-d[2 * i], -d[2 * i + 1]), s[i], both(1.f)), s[i]);
-    const float2 y = mul2(x[i], s[i]);
+    const float2 x = make_float2(clamp_low(z[2 * i], -7.5f), clamp_low(z[2 * i + 1], -7.5f));
+    const float2 v = mul2(x, fma2(mul2(x, x), both(B), both(A)));
+    const float d0 = 1.f + ex2(v.x), d1 = 1.f + ex2(v.y);
+    const float r = rcp(d0 * d1);
+    float2 s = make_float2(r * d1, r * d0);
+    s = fma2(s, fma2(make_float2(-d0, -d1), s, both(1.f)), s);
+    const float2 y = mul2(x, s);
     h[2 * i] = y.x;
     h[2 * i + 1] = y.y;
   }

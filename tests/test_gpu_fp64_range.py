@@ -1,0 +1,41 @@
+"""FP64 transforms of lines far below one (csrc/ps_fix.cuh): the advection of a
+scalar of order one, u . grad theta, is linear in u, so a velocity 2^k times as
+large gives 2^k times the tendency down to where FP64 numbers lose their own
+bits.
+
+Tolerance: FP64 arithmetic rounds at 2^-53 wherever the exponents lie, about 30
+times from the state to the tendency (transforms, products, transforms): 2^-48.
+A subnormal element is off by at most 2^-1075; 2^14 of them against a field of
+norm 2^-1000 add 2^-68.  2^-45 holds both."""
+
+import numpy as np
+import pytest
+
+from paper_1808_01309_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ps():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1808_01309_gb300 import ps as _ps
+    return _ps
+
+
+@pytest.mark.parametrize("n", [(16, 16, 16), (48, 64, 8), (192, 16, 8), (8, 512, 8), (512, 8, 16), (8, 16, 256)], ids=str)
+@pytest.mark.parametrize("k", [-900, -940, -960, -985, -1000])
+def test_advection_by_a_tiny_velocity(ps, k, n):
+    u = inputs.random_solenoidal_field(*n, seed=31, kmax=n)
+    th = inputs.random_scalar_field(*n, seed=32)
+    plan = ps.Plan(*n, prec=ps.Precision.FP64, eq=ps.Equations.BOUSSINESQ, nu=0.0, kappa=0.0, n_bv=0.0)
+
+    def tendency(scale):
+        s = np.concatenate([np.ldexp(u.real, scale) + 1j * np.ldexp(u.imag, scale), th])
+        return plan.rhs(torch.from_numpy(s).cuda()).cpu().numpy()[3]
+
+    one, tiny = tendency(0), tendency(k)
+    back = np.ldexp(tiny.real, -k) + 1j * np.ldexp(tiny.imag, -k)
+    assert np.linalg.norm(back - one) <= 2.0 ** -45 * np.linalg.norm(one)
