@@ -93,9 +93,9 @@ __device__ __forceinline__ void gelu_with_grad(float x, float& h, float& g) {
 // step, and the rest runs two values per instruction, since issue bounds the
 // kernel.  A NaN thus stays within its own sample (one rcp for all four values
 // took it to the other one, and ten 64^3 closure steps 2744 instead of 2721 us).
-// z is clamped at -7.5 so that the product of two
-// and its reciprocal stay normal numbers: there and below the result is
-// -4.0e-18 (1 + tanhf: up to 7.7e-8 off by cancellation).
+// z is clamped at -7.5 so that the product of two and its reciprocal stay normal
+// numbers: there and below the result is -4.0e-18 (1 + tanhf: up to 7.7e-8 off
+// by cancellation).
 __device__ __forceinline__ void gelu4(const float (&z)[4], float (&h)[4]) {
   constexpr float A = -2.f * 0.7978845608028654f * 1.4426950408889634f;  // -2 sqrt(2/pi) log2(e)
   constexpr float B = A * 0.044715f;
