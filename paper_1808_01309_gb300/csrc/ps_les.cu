@@ -1093,7 +1093,6 @@ extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int
   const size_t o_pl = take(sizeof(float) * 9 * Pl);               // LES physical (9 fields)
   const size_t o_nrm = take(sizeof(float) * 12);
   Scratch scratch;
-  ps_status st = PS_OK;
   if (scratch_take(need, &scratch) != cudaSuccess) {
     (void)cudaGetLastError();
     set_last_error("ps_les_training_sample: device allocation failed");
@@ -1158,13 +1157,14 @@ extern "C" ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int
     k_features<<<bl, 256, 0, s>>>(pl, X, A, Pl, nrm);
     e = cudaGetLastError();
   }
+  const cudaError_t es = cudaStreamSynchronize(s);  // the scratch is free again, and what failed on the way shows
+  if (e == cudaSuccess) e = es;
+  scratch_return(scratch, e == cudaSuccess);
   if (e != cudaSuccess) {
     set_last_error(std::string("ps_les_training_sample: ") + cudaGetErrorString(e));
-    st = PS_ERR_CUDA;
+    return PS_ERR_CUDA;
   }
-  const cudaError_t es = cudaStreamSynchronize(s);
-  scratch_return(scratch, e == cudaSuccess && es == cudaSuccess);
-  return st;
+  return PS_OK;
 }
 
 extern "C" ps_status ps_les_filter(int n_dns, const void* uhat_dns, int n_les, int kc, void* uhat_les,
