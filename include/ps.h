@@ -410,7 +410,8 @@ ps_status ps_mlp_adam(float* params, const float* grad, float* m, float* v, int 
  *            detach the closure
  *   norm12 : host doubles mean[5], std[5], s_tau, s_A (std, s_tau, s_A > 0)
  * Grid sizes 16..512 (powers of two, 48, 96, 192).  Allocates the closure
- * scratch on first use (about 29 floats per grid point); synchronises the
+ * scratch on first use (38 to 55 floats per grid point; all of it or, on
+ * PS_ERR_OOM, nothing, and the closure stays as it was); synchronises the
  * plan stream.  PS_ERR_UNSUPPORTED for FP64, MHD or spherical truncation. */
 ps_status ps_plan_set_closure(ps_plan* plan, const float* params, const double* norm12);
 

@@ -1108,14 +1108,26 @@ ps_status ps_plan_set_closure(ps_plan* p, const float* params, const double* nor
   const ps::Geo& g = p->g;
   const size_t P = (size_t)g.nx * g.ny * g.nz, M = (size_t)g.nz * g.ny * g.nh;
   if (!p->les_mem[0]) {
+    // all of the scratch or none of it: a plan with a part would pass null
+    // buffers to its next step
     const size_t rows = (size_t)g.nz * g.ny * g.kxp, zrows = (size_t)g.nz * g.cy * g.kxp;
-    const size_t sizes[7] = {sizeof(float) * PS_MLP_NPARAM, sizeof(float) * 16,
-                             sizeof(float2) * std::max(9 * M, 15 * rows),
-                             sizeof(float) * 9 * P, sizeof(float) * 5 * P, sizeof(float) * 6 * P,
-                             sizeof(float2) * p->sz.cmp};
-    for (int i = 0; i < 7; ++i) PS_CU(cudaMalloc(&p->les_mem[i], sizes[i]), "closure scratch");
-    PS_CU(cudaMalloc(&p->les_mem[9], sizeof(float2) * std::max(15 * zrows, 9 * rows)), "closure scratch");
-    PS_CU(cudaMemsetAsync(p->les_mem[6], 0, sizes[6], p->stream), "closure scratch");
+    const struct {
+      int slot;
+      size_t bytes;
+    } need[] = {{0, sizeof(float) * PS_MLP_NPARAM}, {1, sizeof(float) * 16},
+                {2, sizeof(float2) * std::max(9 * M, 15 * rows)}, {3, sizeof(float) * 9 * P},
+                {4, sizeof(float) * 5 * P}, {5, sizeof(float) * 6 * P}, {6, sizeof(float2) * p->sz.cmp},
+                {9, sizeof(float2) * std::max(15 * zrows, 9 * rows)}};
+    void* got[10] = {};
+    cudaError_t e = cudaSuccess;
+    for (const auto& n : need)
+      if (e == cudaSuccess) e = cudaMalloc(&got[n.slot], n.bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(got[6], 0, need[6].bytes, p->stream);
+    if (e != cudaSuccess) {
+      for (void* b : got) cudaFree(b);
+      return cuda_fail(e, "closure scratch");
+    }
+    for (const auto& n : need) p->les_mem[n.slot] = got[n.slot];
   }
   float h[12];
   for (int i = 0; i < 5; ++i) {

@@ -13,7 +13,7 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1808_01309_gb300", "csrc")
-ILLEGAL_ADDRESS = 700  # cudaErrorIllegalAddress
+OUT_OF_MEMORY, ILLEGAL_ADDRESS = 2, 700  # cudaErrorMemoryAllocation, cudaErrorIllegalAddress
 
 
 @pytest.fixture(scope="module")
@@ -58,6 +58,8 @@ def fake(host_lib, monkeypatch):
     monkeypatch.setattr(ps, "_lib", None)
     f = Fake(ps, ps.load(host_lib))
     f.lib.fake_reset()
+    ps.ps_plan_destroy(ps.ps_plan_create(ps.make_config(8)))  # gives back what an earlier call kept
+    assert f.lib.fake_live() == 0
     yield f
     f.lib.fake_reset()
 
@@ -71,3 +73,31 @@ def test_a_failure_seen_at_the_synchronisation_of_a_sample_is_reported(fake):
     assert fake.lib.fake_live() == 0  # no block is kept after a failure
     fake.lib.fake_reset()  # (a real illegal address ends the context)
     fake.sample()
+
+
+NORM = dict(mean=np.zeros(5), std=np.ones(5), s_tau=1.0, s_A=1.0)
+
+
+def _attach(fake, plan):
+    fake.ps.ps_plan_set_closure(plan, np.zeros(fake.ps.MLP_NPARAM, np.float32).ctypes.data, NORM)
+
+
+@pytest.mark.parametrize("nth", range(1, 9))
+def test_a_closure_that_could_not_be_attached_can_be_attached_later(fake, nth):
+    """An allocation that fails leaves nothing behind, and the next call
+    allocates every buffer."""
+    cfg = fake.ps.make_config(32, nu=1e-3)
+    whole, again = (fake.ps.ps_plan_create(cfg) for _ in range(2))
+    before = fake.lib.fake_live()
+    _attach(fake, whole)
+    need = fake.lib.fake_live() - before
+    fake.fail("cudaMalloc", nth, OUT_OF_MEMORY)
+    with pytest.raises(fake.ps.PsError) as e:
+        _attach(fake, again)
+    assert e.value.status == fake.ps.PS_ERR_OOM
+    assert fake.lib.fake_live() == before + need
+    _attach(fake, again)
+    assert fake.lib.fake_live() == before + 2 * need
+    for plan in (whole, again):
+        fake.ps.ps_plan_destroy(plan)
+    assert fake.lib.fake_live() == 0
