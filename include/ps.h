@@ -445,10 +445,13 @@ ps_status ps_plan_closure_grad_transfer(ps_plan* plan, const float* params, cons
  *             33, 12, 13, 23 (the part of the filtered momentum flux that an
  *             LES truncated at kc does not form itself)
  * n_dns, n_les in {16, 32, 48, 64, 96, 128, 192, 256, 512}, n_les <= n_dns,
- * 1 <= kc <= ceil(n_les/3) - 1.  Its scratch takes about 20 bytes per DNS
- * point; a block of at most 512 MiB stays with the library between calls and
- * is given back when a plan is destroyed or an allocation fails.  Synchronises
- * the stream. */
+ * 1 <= kc <= ceil(n_les/3) - 1.  Its scratch takes
+ * 12 + 48 (kc+1)/n_dns (1 + (2kc+1)/n_dns) bytes per DNS point and 108 bytes
+ * per LES point (19 bytes per DNS point from 256^3 to 64^3 with kc = 21, 147 at
+ * n_les = n_dns with kc = n/3).  A block of at most 512 MiB stays with the
+ * library between calls.  It is given back when a plan (of any size) is
+ * destroyed, and before an allocation of any other call of this library fails;
+ * the caller's own allocator does not know of it.  Synchronises the stream. */
 ps_status ps_les_training_sample(int n_dns, const void* uhat_dns, int n_les, int kc, const double* norm12, float* X,
                                  float* A, float* T, void* cuda_stream);
 

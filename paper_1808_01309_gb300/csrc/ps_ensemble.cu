@@ -217,7 +217,7 @@ ps_status persist_build(ps_ensemble* e, void* const* u, double dt, int nsteps) {
     for (int st = 0; st < nst[i]; ++st) args.push_back(plan_stage_args(e->plans[i], u[i], dt, st, false));
     args.push_back(plan_stage_args(e->plans[i], u[i], dt, 0, true));  // stage 0 with the step statistics
   }
-  if (!e->d_err) ENS_CU(cudaMalloc(&e->d_err, sizeof(int)), "error word");
+  if (!e->d_err) ENS_CU(device_alloc(&e->d_err, sizeof(int)), "error word");
   for (auto& a : args) a.err = e->d_err;
   // each member's pass sequence: per step and stage z-inverse, (energy sum,)
   // y-inverse, x, y-forward, z-forward, update
@@ -295,17 +295,17 @@ ps_status persist_build(ps_ensemble* e, void* const* u, double dt, int nsteps) {
     if (e->d_done) cudaFree(e->d_done);
     e->d_passes = nullptr;
     e->d_done = nullptr;
-    ENS_CU(cudaMalloc(&e->d_passes, passes.size() * sizeof(EnsPass)), "work list");
-    ENS_CU(cudaMalloc(&e->d_done, passes.size() * sizeof(unsigned)), "work counters");
+    ENS_CU(device_alloc(&e->d_passes, passes.size() * sizeof(EnsPass)), "work list");
+    ENS_CU(device_alloc(&e->d_done, passes.size() * sizeof(unsigned)), "work counters");
     e->cap_passes = passes.size();
   }
   if (args.size() > e->cap_args) {
     if (e->d_args) cudaFree(e->d_args);
     e->d_args = nullptr;
-    ENS_CU(cudaMalloc(&e->d_args, args.size() * sizeof(PassArgs)), "stage arguments");
+    ENS_CU(device_alloc(&e->d_args, args.size() * sizeof(PassArgs)), "stage arguments");
     e->cap_args = args.size();
   }
-  if (!e->d_head) ENS_CU(cudaMalloc(&e->d_head, sizeof(unsigned long long)), "ticket counter");
+  if (!e->d_head) ENS_CU(device_alloc(&e->d_head, sizeof(unsigned long long)), "ticket counter");
   ENS_CU(cudaMemcpy(e->d_passes, passes.data(), passes.size() * sizeof(EnsPass), cudaMemcpyHostToDevice), "work list");
   ENS_CU(cudaMemcpy(e->d_args, args.data(), args.size() * sizeof(PassArgs), cudaMemcpyHostToDevice), "stage arguments");
   e->npass = (int)passes.size();
@@ -437,7 +437,7 @@ ps_status batch_capture(ps_ensemble* e, void* const* u, double dt, int nsteps) {
     for (int k = 0; k < M; ++k) sums[k] = plan_view(e->plans[c.members[k]]).stats;
     e->bclasses.push_back(c);  // owned by the ensemble from here (freed by drop_bgraph)
     auto& cc = e->bclasses.back();
-    ENS_CU(cudaMalloc(&cc.d_sum, sums.size() * sizeof(double*)), "batched arguments");
+    ENS_CU(device_alloc(&cc.d_sum, sums.size() * sizeof(double*)), "batched arguments");
     ENS_CU(cudaMemcpy(cc.d_sum, sums.data(), sums.size() * sizeof(double*), cudaMemcpyHostToDevice), "batched arguments");
   }
   const int B = (int)e->bclasses.size();
@@ -636,7 +636,7 @@ ps_status ps_ensemble_tune(ps_ensemble* e, const void* const* uhats, double dt, 
   std::vector<void*> work(m, nullptr);
   ps_status st = PS_OK;
   for (size_t i = 0; i < m && st == PS_OK; ++i) {
-    st = cu(cudaMalloc(&work[i], state_bytes(e->cfgs[i])), "tuning copy");
+    st = cu(device_alloc(&work[i], state_bytes(e->cfgs[i])), "tuning copy");
     if (st == PS_OK)
       st = cu(cudaMemcpyAsync(work[i], uhats[i], state_bytes(e->cfgs[i]), cudaMemcpyDeviceToDevice, e->main),
               "tuning copy");

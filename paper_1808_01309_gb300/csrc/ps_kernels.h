@@ -159,6 +159,16 @@ struct LesScratch {
   float2* extra;        // compact closure term (training)
   float* Arows;         // [P][9] gradient rows (training only)
 };
+// Device memory for the library's own buffers: cudaMalloc, tried once more after
+// the block that ps_les_training_sample keeps was given back (ps_les.cu).
+cudaError_t device_alloc(void** p, size_t bytes);
+template <class T>
+cudaError_t device_alloc(T** p, size_t bytes) {
+  return device_alloc(reinterpret_cast<void**>(p), bytes);
+}
+// Gives that block back; false if there is none.
+bool scratch_trim();
+
 cudaError_t launch_stream_copy(const void* src, void* dst, size_t bytes, int nsm, cudaStream_t s);
 cudaError_t launch_copy_cube(const void* src, void* dst, const Geo& g, int nc, size_t vb, int nsm, cudaStream_t s);
 // The gradient of the stage input a.in through the backward z transform, into

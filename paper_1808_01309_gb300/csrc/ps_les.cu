@@ -991,7 +991,7 @@ __global__ void k_truncate(const V* __restrict__ src, const Geo gs, V* __restric
 // snapshot: one block of at most SCRATCH_KEEP bytes is kept between calls.  A
 // call owns the block it takes (concurrent calls allocate their own) and has
 // synchronised its stream when it returns it; it is given back when a plan is
-// destroyed or an allocation here fails (scratch_trim).
+// destroyed and before any allocation of the library fails (device_alloc).
 constexpr size_t SCRATCH_KEEP = 512ull << 20;
 struct Scratch {
   void* p = nullptr;
@@ -1019,7 +1019,7 @@ cudaError_t scratch_take(size_t bytes, Scratch* out) {
   cudaFree(k.p);
   out->bytes = bytes;
   out->device = dev;
-  return cudaMalloc(&out->p, bytes);
+  return device_alloc(&out->p, bytes);
 }
 // ok: nothing the call launched is still running or has failed.
 void scratch_return(const Scratch& s, bool ok) {
@@ -1050,7 +1050,19 @@ unsigned blocks(long long n) { return (unsigned)((n + 255) / 256); }
 
 }  // namespace les
 
-void scratch_trim() { cudaFree(les::scratch_kept_out().p); }
+bool scratch_trim() {
+  void* p = les::scratch_kept_out().p;
+  cudaFree(p);
+  return p != nullptr;
+}
+cudaError_t device_alloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && scratch_trim()) {
+    (void)cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
 
 }  // namespace ps
 
@@ -1220,8 +1232,8 @@ ps_status fft_run(int n, int nfields, const void* in, void* out, void* cuda_stre
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   V* tw = nullptr;
   V* spec = nullptr;
-  cudaError_t e = cudaMalloc(&tw, sizeof(V) * n);
-  if (e == cudaSuccess && backward) e = cudaMalloc(&spec, sizeof(V) * nfields * M);  // the z, y passes work in place
+  cudaError_t e = device_alloc(&tw, sizeof(V) * n);
+  if (e == cudaSuccess && backward) e = device_alloc(&spec, sizeof(V) * nfields * M);  // the z, y passes work in place
   if (e != cudaSuccess) {
     cudaFree(tw);
     (void)cudaGetLastError();

@@ -137,8 +137,6 @@ struct TimedLaunch {
 namespace ps {
 // Lets other translation units of the library report through ps_last_error().
 void set_last_error(const std::string& msg) { g_last_error = msg; }
-// Gives back the scratch block kept by ps_les_training_sample (ps_les.cu).
-void scratch_trim();
 }  // namespace ps
 
 struct ps_plan {
@@ -500,7 +498,7 @@ ps_status setup_forcing(ps_plan* p) {
   p->Fy = ext[1];
   p->Fz = ext[2];
   const size_t n = 3ull * (p->Fx + 1) * (2 * p->Fy + 1) * (2 * p->Fz + 1);
-  PS_CU(cudaMalloc(&p->fbox, n * p->sz.vb), "forcing box");
+  PS_CU(ps::device_alloc(&p->fbox, n * p->sz.vb), "forcing box");
   PS_CU(launch_forcing_gather<T>(p->g, f, p->Fx, p->Fy, p->Fz, p->fbox, p->stream), "forcing gather");
   PS_CU(cudaStreamSynchronize(p->stream), "forcing gather");
   return PS_OK;
@@ -666,12 +664,7 @@ ps_status ps_plan_create(const ps_config* cfg, void* cuda_stream, ps_plan** out)
   const size_t vb = p->sz.vb, tb = cfg->prec == PS_FP32 ? 4 : 8;
 #define ALLOC(ptr, bytes, what)                          \
   do {                                                   \
-    cudaError_t e_ = cudaMalloc((void**)&(ptr), (bytes)); \
-    if (e_ == cudaErrorMemoryAllocation) {               \
-      (void)cudaGetLastError();                          \
-      ps::scratch_trim();                                \
-      e_ = cudaMalloc((void**)&(ptr), (bytes));          \
-    }                                                    \
+    cudaError_t e_ = ps::device_alloc(&(ptr), (bytes));  \
     if (e_ != cudaSuccess) return bail(cuda_fail(e_, what)); \
   } while (0)
   ALLOC(p->a6, p->sz.a6 * vb, "scratch a");
@@ -933,7 +926,7 @@ ps_status ps_rk_step_host(ps_plan* p, void* uhat_host, double dt, double t, int 
     PS_CU(cudaStreamSynchronize(p->stream), "host-path sync");
     return check_device_error(p);
   }
-  if (!p->hstate) PS_CU(cudaMalloc(&p->hstate, bytes), "host-path state");
+  if (!p->hstate) PS_CU(ps::device_alloc(&p->hstate, bytes), "host-path state");
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
   const bool cube = mapped && (p->host_mode == PS_HOST_AUTO || p->host_mode == PS_HOST_CUBE_CE);
@@ -950,7 +943,7 @@ ps_status ps_rk_step_host(ps_plan* p, void* uhat_host, double dt, double t, int 
       PS_CU(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking), "side stream");
       PS_CU(cudaEventCreateWithFlags(&p->side_go, cudaEventDisableTiming), "side event");
       PS_CU(cudaEventCreateWithFlags(&p->side_done, cudaEventDisableTiming), "side event");
-      PS_CU(cudaMalloc(&p->zbuf, ZBUF_BYTES), "zero buffer");
+      PS_CU(ps::device_alloc(&p->zbuf, ZBUF_BYTES), "zero buffer");
       PS_CU(cudaMemsetAsync(p->zbuf, 0, ZBUF_BYTES, p->stream), "zero buffer");
     }
     PS_CU(cudaEventRecord(p->side_go, p->stream), "side event");
@@ -1121,7 +1114,7 @@ ps_status ps_plan_set_closure(ps_plan* p, const float* params, const double* nor
     void* got[10] = {};
     cudaError_t e = cudaSuccess;
     for (const auto& n : need)
-      if (e == cudaSuccess) e = cudaMalloc(&got[n.slot], n.bytes);
+      if (e == cudaSuccess) e = ps::device_alloc(&got[n.slot], n.bytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(got[6], 0, need[6].bytes, p->stream);
     if (e != cudaSuccess) {
       for (void* b : got) cudaFree(b);
@@ -1160,7 +1153,7 @@ ps_status ps_plan_closure_grad(ps_plan* p, const float* params, const void* ubar
   DeviceGuard dg(p->device);
   const ps::Geo& g = p->g;
   const size_t P = (size_t)g.nx * g.ny * g.nz;
-  if (!p->les_mem[7]) PS_CU(cudaMalloc(&p->les_mem[7], sizeof(float) * 9 * P), "closure training scratch");
+  if (!p->les_mem[7]) PS_CU(ps::device_alloc(&p->les_mem[7], sizeof(float) * 9 * P), "closure training scratch");
   p->les.Arows = static_cast<float*>(p->les_mem[7]);
   if (!accumulate) {
     PS_CU(cudaMemsetAsync(grad, 0, sizeof(float) * PS_MLP_NPARAM, p->stream), "gradient reset");
@@ -1182,8 +1175,8 @@ ps_status ps_plan_closure_grad_transfer(ps_plan* p, const float* params, const v
   DeviceGuard dg(p->device);
   const ps::Geo& g = p->g;
   const size_t P = (size_t)g.nx * g.ny * g.nz;
-  if (!p->les_mem[7]) PS_CU(cudaMalloc(&p->les_mem[7], sizeof(float) * 9 * P), "closure training scratch");
-  if (!p->les_mem[8]) PS_CU(cudaMalloc(&p->les_mem[8], sizeof(double) * 3 * 1024), "closure transfer scratch");
+  if (!p->les_mem[7]) PS_CU(ps::device_alloc(&p->les_mem[7], sizeof(float) * 9 * P), "closure training scratch");
+  if (!p->les_mem[8]) PS_CU(ps::device_alloc(&p->les_mem[8], sizeof(double) * 3 * 1024), "closure transfer scratch");
   p->les.Arows = static_cast<float*>(p->les_mem[7]);
   double* te = static_cast<double*>(p->les_mem[8]);
   PS_CU(cudaMemcpyAsync(te, t_exact, sizeof(double) * nshells, cudaMemcpyHostToDevice, p->stream), "transfer target");
@@ -1310,12 +1303,12 @@ ps_status ps_slab_create(const ps_config* cfg, int kx_lo, int kx_hi, int z_lo, i
   };
   cudaError_t e;
   const size_t a6 = std::max(6ull * g.nz * g.cy * kxp, 3ull * g.cz * g.cy * kxp);
-  if ((e = cudaMalloc(&s->a6, a6 * s->vb)) != cudaSuccess) return bail(cuda_fail(e, "slab scratch"));
-  if ((e = cudaMalloc(&s->b6, 3ull * g.nz * g.cy * kxp * s->vb)) != cudaSuccess)
+  if ((e = ps::device_alloc(&s->a6, a6 * s->vb)) != cudaSuccess) return bail(cuda_fail(e, "slab scratch"));
+  if ((e = ps::device_alloc(&s->b6, 3ull * g.nz * g.cy * kxp * s->vb)) != cudaSuccess)
     return bail(cuda_fail(e, "slab scratch"));
-  if ((e = cudaMalloc(&s->tw, (size_t)(g.nx + g.ny + g.nz) * s->vb)) != cudaSuccess)
+  if ((e = ps::device_alloc(&s->tw, (size_t)(g.nx + g.ny + g.nz) * s->vb)) != cudaSuccess)
     return bail(cuda_fail(e, "slab twiddles"));
-  if ((e = cudaMalloc(&s->err, sizeof(int))) != cudaSuccess) return bail(cuda_fail(e, "slab error word"));
+  if ((e = ps::device_alloc(&s->err, sizeof(int))) != cudaSuccess) return bail(cuda_fail(e, "slab error word"));
   if ((e = cudaMemsetAsync(s->err, 0, sizeof(int), s->stream)) != cudaSuccess)
     return bail(cuda_fail(e, "slab error word"));
   if (cfg->prec == PS_FP32) {
@@ -1335,7 +1328,7 @@ ps_status ps_slab_create(const ps_config* cfg, int kx_lo, int kx_hi, int z_lo, i
   if (cfg->forcing) {
     // the whole local retained block as the forcing box
     const size_t n = 3ull * s->gl.ncx * g.cy * g.cz;
-    if ((e = cudaMalloc(&s->fbox, n * s->vb)) != cudaSuccess) return bail(cuda_fail(e, "slab forcing box"));
+    if ((e = ps::device_alloc(&s->fbox, n * s->vb)) != cudaSuccess) return bail(cuda_fail(e, "slab forcing box"));
     const Spec f = local_spec(s->gl, cfg->forcing);
     e = cfg->prec == PS_FP32 ? launch_forcing_gather<float>(s->gl, f, s->gl.ncx - 1, g.Ky, g.Kz, s->fbox, s->stream)
                              : launch_forcing_gather<double>(s->gl, f, s->gl.ncx - 1, g.Ky, g.Kz, s->fbox, s->stream);

@@ -101,3 +101,80 @@ def test_a_closure_that_could_not_be_attached_can_be_attached_later(fake, nth):
     for plan in (whole, again):
         fake.ps.ps_plan_destroy(plan)
     assert fake.lib.fake_live() == 0
+
+
+class Calls:
+    """Calls that allocate device memory, each on objects made beforehand."""
+
+    def __init__(self, fake):
+        self.ps, self.fake, self.made = fake.ps, fake, []
+        self.n = 32
+        self.u = np.zeros((3, 32, 32, 17), np.complex64)
+        self.f = np.ones_like(self.u)
+        self.vec, self.loss = np.zeros(fake.ps.MLP_NPARAM, np.float32), np.zeros(1)
+
+    def plan(self):
+        self.made.append((self.ps.ps_plan_destroy, self.ps.ps_plan_create(self.ps.make_config(self.n, nu=1e-3))))
+        return self.made[-1][1]
+
+    def close(self):
+        for destroy, handle in reversed(self.made):
+            destroy(handle)
+        self.made = []
+
+    def prepare(self, name):
+        """The objects of one call; returns the call."""
+        ps, u, vec = self.ps, self.u.ctypes.data, self.vec.ctypes.data
+        if name == "plan":
+            return self.plan
+        if name in ("closure", "closure gradient", "closure transfer"):
+            p = self.plan()
+            if name == "closure":
+                return lambda: _attach(self.fake, p)
+            _attach(self.fake, p)
+            if name == "closure gradient":
+                return lambda: ps.ps_plan_closure_grad(p, vec, u, self.f.ctypes.data, vec, self.loss.ctypes.data)
+            return lambda: ps.ps_plan_closure_grad_transfer(p, vec, u, np.zeros(8), vec, self.loss.ctypes.data)
+        if name in ("host step", "host step, copy engines"):
+            p = self.plan()
+            ps.ps_plan_set_host_mode(p, ps.HOST_AUTO if name == "host step" else ps.HOST_CUBE_CE)
+            return lambda: ps.ps_rk_step_host(p, u, 1e-3)
+        if name == "slab":
+            cfg = ps.make_config(self.n, nu=1e-3, forcing=self.f.ctypes.data)
+            return lambda: self.made.append((ps.ps_slab_destroy, ps.ps_slab_create(cfg, 0, 6, 0, 16)))
+        if name == "backward transform":
+            return lambda: ps.ps_fft_c2r(self.n, 3, u, np.zeros((3, 32, 32, 32), np.float32).ctypes.data)
+        if name == "sample":
+            return lambda: self.fake.sample(64, 32, 10)
+        e = ps.ps_ensemble_create([ps.make_config(self.n, nu=1e-3) for _ in range(2)])
+        self.made.append((ps.ps_ensemble_destroy, e))
+        states = [self.u.ctypes.data] * 2
+        if name == "ensemble tuning":
+            return lambda: ps.ps_ensemble_tune(e, states, 1e-3)
+        mode = ps.ENS_PERSISTENT if name == "persistent ensemble" else ps.ENS_BATCHED
+        return lambda: ps.ps_ensemble_rk_steps(e, states, 1e-3, 0.0, 2, mode)
+
+
+@pytest.mark.parametrize("name", ["plan", "closure", "closure gradient", "closure transfer", "host step",
+                                  "host step, copy engines", "slab", "backward transform", "sample",
+                                  "persistent ensemble", "batched ensemble", "ensemble tuning"])
+def test_a_call_that_fits_without_the_kept_scratch_fits_with_it(fake, name):
+    """Memory for a call, and no more: the block that a training sample left is
+    given back to it."""
+    calls = Calls(fake)
+    call = calls.prepare(name)
+    fake.lib.fake_reset()
+    call()
+    need = fake.lib.fake_peak()
+    calls.close()
+    fake.ps.ps_plan_destroy(fake.ps.ps_plan_create(fake.ps.make_config(8)))
+    assert fake.lib.fake_live() == 0
+    call = calls.prepare(name)
+    before = fake.lib.fake_live()
+    fake.sample()
+    assert fake.lib.fake_live() > before  # a block is kept
+    fake.lib.fake_budget(need)
+    try:
+        call()
+    finally:
+        calls.close()
