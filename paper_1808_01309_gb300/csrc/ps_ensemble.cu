@@ -295,6 +295,7 @@ ps_status persist_build(ps_ensemble* e, void* const* u, double dt, int nsteps) {
     if (e->d_done) cudaFree(e->d_done);
     e->d_passes = nullptr;
     e->d_done = nullptr;
+    e->cap_passes = 0;  // until both are there
     ENS_CU(device_alloc(&e->d_passes, passes.size() * sizeof(EnsPass)), "work list");
     ENS_CU(device_alloc(&e->d_done, passes.size() * sizeof(unsigned)), "work counters");
     e->cap_passes = passes.size();
@@ -302,6 +303,7 @@ ps_status persist_build(ps_ensemble* e, void* const* u, double dt, int nsteps) {
   if (args.size() > e->cap_args) {
     if (e->d_args) cudaFree(e->d_args);
     e->d_args = nullptr;
+    e->cap_args = 0;
     ENS_CU(device_alloc(&e->d_args, args.size() * sizeof(PassArgs)), "stage arguments");
     e->cap_args = args.size();
   }

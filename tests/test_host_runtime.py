@@ -178,3 +178,19 @@ def test_a_call_that_fits_without_the_kept_scratch_fits_with_it(fake, name):
         call()
     finally:
         calls.close()
+
+
+@pytest.mark.parametrize("nth", [1, 2])
+def test_a_persistent_ensemble_recovers_from_a_work_list_that_did_not_fit(fake, nth):
+    calls = Calls(fake)
+    call = calls.prepare("persistent ensemble")
+    e, states = calls.made[-1][1], [calls.u.ctypes.data] * 2
+    call()  # two steps: a list of that size
+    fake.fail("cudaMalloc", nth, OUT_OF_MEMORY)
+    with pytest.raises(fake.ps.PsError) as err:
+        fake.ps.ps_ensemble_rk_steps(e, states, 1e-3, 0.0, 5, fake.ps.ENS_PERSISTENT)
+    assert err.value.status == fake.ps.PS_ERR_OOM
+    fake.lib.fake_reset()
+    call()
+    calls.close()
+    assert fake.lib.fake_live() == 0
