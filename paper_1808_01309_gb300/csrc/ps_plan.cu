@@ -939,12 +939,16 @@ ps_status ps_rk_step_host(ps_plan* p, void* uhat_host, double dt, double t, int 
   } else if (cube) {
     // only the retained modes cross the host link; the masked modes of the
     // host state are zeroed by copy engines while the steps run
-    if (!p->side) {
-      PS_CU(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking), "side stream");
-      PS_CU(cudaEventCreateWithFlags(&p->side_go, cudaEventDisableTiming), "side event");
-      PS_CU(cudaEventCreateWithFlags(&p->side_done, cudaEventDisableTiming), "side event");
-      PS_CU(ps::device_alloc(&p->zbuf, ZBUF_BYTES), "zero buffer");
-      PS_CU(cudaMemsetAsync(p->zbuf, 0, ZBUF_BYTES, p->stream), "zero buffer");
+    if (!p->side) PS_CU(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking), "side stream");
+    if (!p->side_go) PS_CU(cudaEventCreateWithFlags(&p->side_go, cudaEventDisableTiming), "side event");
+    if (!p->side_done) PS_CU(cudaEventCreateWithFlags(&p->side_done, cudaEventDisableTiming), "side event");
+    if (!p->zbuf) {
+      void* z = nullptr;
+      PS_CU(ps::device_alloc(&z, ZBUF_BYTES), "zero buffer");
+      const cudaError_t e = cudaMemsetAsync(z, 0, ZBUF_BYTES, p->stream);
+      if (e != cudaSuccess) cudaFree(z);
+      PS_CU(e, "zero buffer");
+      p->zbuf = z;
     }
     PS_CU(cudaEventRecord(p->side_go, p->stream), "side event");
     PS_CU(cudaStreamWaitEvent(p->side, p->side_go, 0), "side event");

@@ -194,3 +194,16 @@ def test_a_persistent_ensemble_recovers_from_a_work_list_that_did_not_fit(fake, 
     call()
     calls.close()
     assert fake.lib.fake_live() == 0
+
+
+def test_a_host_step_recovers_from_a_zero_buffer_that_did_not_fit(fake):
+    calls = Calls(fake)
+    call = calls.prepare("host step, copy engines")
+    fake.fail("cudaMalloc", 2, OUT_OF_MEMORY)  # (the first is the device state)
+    with pytest.raises(fake.ps.PsError) as err:
+        call()
+    assert err.value.status == fake.ps.PS_ERR_OOM
+    fake.lib.fake_reset()
+    call()
+    calls.close()
+    assert fake.lib.fake_live() == 0
