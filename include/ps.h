@@ -338,13 +338,14 @@ ps_status ps_ensemble_destroy(ps_ensemble* e);
 ps_status ps_ensemble_rk_steps(ps_ensemble* e, void* const* uhats, double dt, double t, int nsteps,
                                ps_ens_mode mode);
 
-/* Autotuner: times, on device copies of uhats (left unchanged), for each
- * distinct grid the x-pass rows per CTA and the tile shape (columns per CTA,
- * radix schedule) of each column pass, then the number of concurrent graph
- * branches, the persistent launch's knobs and the members per batched
- * launch; keeps the fastest of each, sets the mode PS_ENS_AUTO runs and
- * reports them.  Allocates temporary copies of the states.  Synchronises
- * the ensemble stream. */
+/* Autotuner, on device copies of uhats (left unchanged): times the number of
+ * concurrent graph branches; then, for each distinct grid, the x-pass rows per
+ * CTA and the tile shape (columns per CTA, radix schedule) of each column pass,
+ * on the grid's first member with the launches that a graph of that many
+ * branches makes, kept if the graph of all members gains; then the persistent
+ * launch's knobs and the members per batched launch.  Keeps the fastest of each,
+ * sets the mode PS_ENS_AUTO runs and reports them.  Allocates temporary copies
+ * of the states.  Synchronises the ensemble stream. */
 ps_status ps_ensemble_tune(ps_ensemble* e, const void* const* uhats, double dt, ps_ens_tuning* out);
 
 /* Synchronises the ensemble stream and reports whether a bounded device wait

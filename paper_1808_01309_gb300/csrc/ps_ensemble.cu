@@ -114,10 +114,7 @@ void drop_graph(ps_ensemble* e) {
 
 // Sequential: every member's steps on the ensemble stream, member by member.
 ps_status run_sequential(ps_ensemble* e, void* const* u, double dt, double t, int nsteps) {
-  for (size_t i = 0; i < e->plans.size(); ++i) {
-    plan_set_stream(e->plans[i], e->main);
-    plan_set_beside(e->plans[i], 1);
-  }
+  for (size_t i = 0; i < e->plans.size(); ++i) plan_set_stream(e->plans[i], e->main);
   for (int s = 0; s < nsteps; ++s)
     for (size_t i = 0; i < e->plans.size(); ++i) {
       ps_status st = ps_rk_step(e->plans[i], u[i], dt, t + s * dt);
@@ -151,6 +148,7 @@ ps_status capture(ps_ensemble* e, void* const* u, double dt, double t, int nstep
   }
   cudaGraph_t g = nullptr;
   ce = cudaStreamEndCapture(e->cap, &g);
+  for (ps_plan* p : e->plans) plan_set_beside(p, 1);
   if (st != PS_OK) {
     if (g) cudaGraphDestroy(g);
     return st;
@@ -644,25 +642,61 @@ ps_status ps_ensemble_tune(ps_ensemble* e, const void* const* uhats, double dt, 
               "tuning copy");
   }
   *out = ps_ens_tuning{};
-  // 1. x-pass rows per CTA, per distinct grid (timed on its first member)
-  std::vector<int> done;
+  const auto default_shapes = [&] {
+    for (ps_plan* p : e->plans) {
+      plan_set_xrpc(p, 0);
+      for (int k = 0; k < 3; ++k) plan_set_shape(p, k, 0);
+    }
+  };
+  default_shapes();
+  drop_graph(e);
+  const auto time_graph = [&](double* ms) {
+    return time_ms(e, 3, [&] { return run_graph(e, work.data(), dt, 0.0, 1); }, ms);
+  };
+  // 1. number of concurrent graph branches, timed on one step of all members
+  if (st == PS_OK) {
+    const int cand[] = {1, 2, 4, 8, 16, 24, 32, 48, 64};
+    double best = 1e30;
+    int best_b = 1;
+    for (int b : cand) {
+      if (b > (int)m) break;
+      e->nbranch = b;
+      double ms = 0;
+      st = time_graph(&ms);
+      if (st != PS_OK) break;
+      if (ms < best * 0.98) {
+        best = ms;
+        best_b = b;
+      }
+    }
+    e->nbranch = best_b;
+    out->branches = best_b;
+    out->step_ms = best;
+  }
+  // 2. x-pass rows per CTA and tile shapes per distinct grid, timed on its first
+  //    member with the launches that a graph of that many branches makes of it
+  //    (the launchers' rules depend on the launches beside: PassArgs::beside)
+  std::vector<int> first;  // first member of each distinct grid
+  bool shaped = false;
   for (size_t i = 0; i < m && st == PS_OK; ++i) {
     const ps_config& c = e->cfgs[i];
-    bool seen = false;
-    for (int j : done) {
-      const ps_config& d = e->cfgs[j];
-      seen |= d.nx == c.nx && d.ny == c.ny && d.nz == c.nz && d.prec == c.prec;
-    }
-    if (seen) continue;
-    done.push_back((int)i);
+    const auto same_grid = [&](const ps_config& d) {
+      return d.nx == c.nx && d.ny == c.ny && d.nz == c.nz && d.prec == c.prec;
+    };
+    if (std::any_of(first.begin(), first.end(), [&](int j) { return same_grid(e->cfgs[j]); })) continue;
+    first.push_back((int)i);
     const int cand[] = {0, 16, 8, 4, 2, 1};
     double best = 1e30;
     int best_r = 0;
     plan_set_stream(e->plans[i], e->main);
+    plan_set_beside(e->plans[i], e->nbranch);
+    const auto time_step = [&](double* ms) {
+      return time_ms(e, 3, [&] { return ps_rk_step(e->plans[i], work[i], dt, 0.0); }, ms);
+    };
     for (int r : cand) {
       plan_set_xrpc(e->plans[i], r);
       double ms = 0;
-      st = time_ms(e, 3, [&] { return ps_rk_step(e->plans[i], work[i], dt, 0.0); }, &ms);
+      st = time_step(&ms);
       if (st != PS_OK) break;
       if (ms < best * 0.98) {
         best = ms;
@@ -677,56 +711,44 @@ ps_status ps_ensemble_tune(ps_ensemble* e, const void* const* uhats, double dt, 
       for (int var = 1; var <= 2 && st == PS_OK; ++var) {
         if (!plan_set_shape(e->plans[i], k, var)) continue;
         double ms = 0;
-        st = time_ms(e, 3, [&] { return ps_rk_step(e->plans[i], work[i], dt, 0.0); }, &ms);
+        st = time_step(&ms);
         if (st == PS_OK && ms < best * 0.98) {
           best = ms;
           best_var[k] = var;
         }
         plan_set_shape(e->plans[i], k, best_var[k]);
       }
-    for (size_t j = i; j < m; ++j) {
-      const ps_config& d = e->cfgs[j];
-      if (d.nx == c.nx && d.ny == c.ny && d.nz == c.nz && d.prec == c.prec) {
+    plan_set_beside(e->plans[i], 1);
+    for (size_t j = i; j < m; ++j)
+      if (same_grid(e->cfgs[j])) {
         plan_set_xrpc(e->plans[j], best_r);
         for (int k = 0; k < 3; ++k) plan_set_shape(e->plans[j], k, best_var[k]);
       }
-    }
-    if (out->nsizes < PS_ENS_MAX_SIZES) {
-      const int z = out->nsizes;
-      out->n[z] = c.nx;
-      out->xrpc[z] = best_r;
-      for (int k = 0; k < 3; ++k) {
-        const int len = k == 1 ? c.ny : c.nz;
-        int cols = 0, pts = 0;
-        if (c.prec == PS_FP32) pass_shape<float>(k, len, best_var[k], &cols, &pts);
-        else pass_shape<double>(k, len, best_var[k], &cols, &pts);
-        out->pass_cols[z][k] = cols;
-        out->pass_points[z][k] = pts;
-      }
-      out->nsizes++;
-    }
+    shaped |= best_r || best_var[0] || best_var[1] || best_var[2];
   }
-  // 2. number of concurrent graph branches, timed on one step of all members
-  if (st == PS_OK) {
-    const int cand[] = {1, 2, 4, 8, 16, 24, 32, 48, 64};
-    double best = 1e30;
-    int best_b = 1;
-    for (int b : cand) {
-      if (b > (int)m) break;
-      e->nbranch = b;
-      double ms = 0;
-      st = time_ms(e, 3, [&] { return run_graph(e, work.data(), dt, 0.0, 1); }, &ms);
-      if (st != PS_OK) break;
-      if (ms < best * 0.98) {
-        best = ms;
-        best_b = b;
-      }
-    }
-    e->nbranch = best_b;
-    out->branches = best_b;
-    out->step_ms = best;
+  // what gains on one plan alone is kept if all members gain together
+  if (st == PS_OK && shaped) {
+    double ms = 0;
+    drop_graph(e);
+    st = time_graph(&ms);
+    if (st == PS_OK && ms < out->step_ms) out->step_ms = ms;
+    else default_shapes();
   }
   drop_graph(e);
+  for (size_t f = 0; f < first.size() && out->nsizes < PS_ENS_MAX_SIZES && st == PS_OK; ++f) {
+    const ps_config& c = e->cfgs[first[f]];
+    const int z = out->nsizes++;
+    out->n[z] = c.nx;
+    out->xrpc[z] = plan_xrpc(e->plans[first[f]]);
+    for (int k = 0; k < 3; ++k) {
+      const int len = k == 1 ? c.ny : c.nz, var = plan_shape(e->plans[first[f]], k);
+      int cols = 0, pts = 0;
+      if (c.prec == PS_FP32) pass_shape<float>(k, len, var, &cols, &pts);
+      else pass_shape<double>(k, len, var, &cols, &pts);
+      out->pass_cols[z][k] = cols;
+      out->pass_points[z][k] = pts;
+    }
+  }
   // 3. persistent launch: CTAs per SM, member order and tiles per work item
   //    per pass kind, one knob at a time (coordinate descent), each candidate
   //    timed on one step of all members

@@ -190,6 +190,7 @@ cudaError_t les_closure_grad(const Geo& g, Spec in, Spec f, const void* twx, con
 void plan_set_stream(struct ::ps_plan* p, cudaStream_t s);
 cudaStream_t plan_stream(const struct ::ps_plan* p);
 void plan_set_xrpc(struct ::ps_plan* p, int rpc);
+int plan_xrpc(const struct ::ps_plan* p);
 // Launches of other plans that run beside p's, p's included (PassArgs::beside).
 void plan_set_beside(struct ::ps_plan* p, int n);
 // Forget the cached integrating-factor tables so the next step recomputes them

@@ -542,6 +542,7 @@ namespace ps {
 void plan_set_stream(ps_plan* p, cudaStream_t s) { p->stream = s; }
 cudaStream_t plan_stream(const ps_plan* p) { return p->stream; }
 void plan_set_beside(ps_plan* p, int n) { p->beside = n; }
+int plan_xrpc(const ps_plan* p) { return p->xrpc; }
 void plan_set_xrpc(ps_plan* p, int rpc) {
   if (p->xrpc != rpc) drop_cached_graph(p);
   p->xrpc = rpc;

@@ -207,3 +207,42 @@ def test_a_host_step_recovers_from_a_zero_buffer_that_did_not_fit(fake):
     call()
     calls.close()
     assert fake.lib.fake_live() == 0
+
+
+def _launches(fake, captured):
+    """(kernel, grid, block, shared memory) of the passes launched in or out of a capture."""
+    rows = [line.rsplit(" ", 1) for line in fake.lib.fake_launches().decode().splitlines()]
+    kinds = ("k_zinv", "k_yinv", "k_xpass", "k_yfwd", "k_zfwd")
+    return [what for what, flag in rows if flag == str(int(captured)) and any(k in what for k in kinds)]
+
+
+@pytest.mark.parametrize("sizes", [(32, 32), (64, 64, 64, 64), (128, 64, 128, 64)], ids=str)
+def test_the_ensemble_tuner_times_the_kernels_that_the_graph_runs(fake, sizes):
+    """Where the tuner keeps the default shapes, what it timed plan by plan is
+    what the graph launches, and a second tuning times the same again."""
+    ps = fake.ps
+    e = ps.ps_ensemble_create([ps.make_config(n, nu=1e-3) for n in sizes])
+    states = [np.zeros((3, n, n, n // 2 + 1), np.complex64) for n in sizes]
+    ptrs = [s.ctypes.data for s in states]
+    timed = []
+    for _ in range(2):
+        fake.lib.fake_reset()
+        tuning = ps.ps_ensemble_tune(e, ptrs, 1e-3)
+        assert tuning["branches"] == len(sizes) and not any(tuning["xrpc"].values())
+        timed.append(_launches(fake, False))
+    assert timed[0] == timed[1]
+    fake.lib.fake_reset()
+    ps.ps_ensemble_rk_steps(e, ptrs, 1e-3, 0.0, 1, ps.ENS_GRAPH)
+    run = set(_launches(fake, True))
+    assert len(run) == 5 * len(set(sizes)) and run <= set(timed[0])
+    # and a member stepped alone afterwards takes the launches of a plan alone
+    fake.lib.fake_reset()
+    ps.ps_ensemble_rk_steps(e, ptrs, 1e-3, 0.0, 1, ps.ENS_SEQUENTIAL)
+    alone = set(_launches(fake, False))
+    fake.lib.fake_reset()
+    for n, s in zip(sizes, ptrs):
+        plan = ps.ps_plan_create(ps.make_config(n, nu=1e-3))
+        ps.ps_rk_step(plan, s, 1e-3)
+        ps.ps_plan_destroy(plan)
+    assert alone == set(_launches(fake, False))
+    ps.ps_ensemble_destroy(e)
