@@ -655,11 +655,15 @@ ps_status ps_ensemble_tune(ps_ensemble* e, const void* const* uhats, double dt, 
   };
   // 1. number of concurrent graph branches, timed on one step of all members
   if (st == PS_OK) {
+    // up to one per member: 12 members (32^3 to 96^3) 0.54 ms a step with 12
+    // branches, the untuned count, 0.65 with 8
     const int cand[] = {1, 2, 4, 8, 16, 24, 32, 48, 64};
     double best = 1e30;
-    int best_b = 1;
-    for (int b : cand) {
-      if (b > (int)m) break;
+    int best_b = 1, last = 0;
+    for (int c : cand) {
+      const int b = std::min(c, (int)m);
+      if (b == last) break;
+      last = b;
       e->nbranch = b;
       double ms = 0;
       st = time_graph(&ms);

@@ -216,10 +216,11 @@ def _launches(fake, captured):
     return [what for what, flag in rows if flag == str(int(captured)) and any(k in what for k in kinds)]
 
 
-@pytest.mark.parametrize("sizes", [(32, 32), (64, 64, 64, 64), (128, 64, 128, 64)], ids=str)
+@pytest.mark.parametrize("sizes", [(32, 32), (64,) * 3, (64,) * 12, (128, 64, 128, 64)], ids=str)
 def test_the_ensemble_tuner_times_the_kernels_that_the_graph_runs(fake, sizes):
     """Where the tuner keeps the default shapes, what it timed plan by plan is
-    what the graph launches, and a second tuning times the same again."""
+    what the graph launches, and a second tuning times the same again.  A branch
+    per member is among the branch counts."""
     ps = fake.ps
     e = ps.ps_ensemble_create([ps.make_config(n, nu=1e-3) for n in sizes])
     states = [np.zeros((3, n, n, n // 2 + 1), np.complex64) for n in sizes]
