@@ -83,7 +83,14 @@ typedef struct ps_plan ps_plan;
 /* One solve (Sec. 2: grid and box may differ per axis).
  *   nx, ny, nz : powers of two in [8, 1024], or 48, 96, 192 (radix-3 lines)
  *   lx, ly, lz : box lengths, finite and > 0
- *   prec       : arithmetic and storage precision of all fields
+ *   prec       : arithmetic and storage precision of all fields.  PS_FP64 line
+ *                transforms run in block fixed point: with S the sum of
+ *                |re| + |im| over a line along an axis, each element is held to
+ *                2^-61 S, which an FP64 transform's own rounding reaches at
+ *                512 points, but to no less than 2^-1021: lines with S below
+ *                2^-937 (1e-282) lose bits.  A line with an Inf or a NaN, or
+ *                with S from 2^1024 on, becomes NaN as a whole; the sign of a
+ *                zero is not kept
  *   eq         : PS_HD, or PS_MHD (Eqs. uMHD, bMHD: the state then has six
  *                components u_x, u_y, u_z, B_x, B_y, B_z; the magnetic
  *                field advances with dB/dt = curl(u x B) - eta |k|^2 B,

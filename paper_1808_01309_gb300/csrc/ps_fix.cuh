@@ -17,11 +17,14 @@
 // intermediate at every operation); twiddles carry 62 bits instead of 53.
 // Measured against 80-bit transforms (right-hand side without diffusion, 64^3,
 // 96x48x64, 256x16x128, 512x16x16): relative L2 error 2.6e-16 to 2.7e-16, with
-// FP64 transforms 5.4e-16 to 6.2e-16.  256^3 RK4 step: 35.4 -> 14.0 ms.
+// FP64 transforms 5.4e-16 to 6.2e-16.  256^3 RK4 step: 35.4 -> 14.0 ms (10.7 with
+// the x pass one line at a time, ps_passes.cuh).
 //
 // Range: a line with an Inf or a NaN (or whose L1 overflows) becomes NaN as a
 // whole; a line whose L1 is below 2^-937 loses bits (the scale is capped at
-// 2^1021), zero lines stay zero.
+// 2^1021, so that results need no gradual underflow), zero lines stay zero.
+// Scaling such lines by 2^512 and back, with a branch per line, restored them at
+// 2 to 9 % of every FP64 right-hand side (128^3: 338 -> 356 us).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
