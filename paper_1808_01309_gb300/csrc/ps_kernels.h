@@ -84,7 +84,7 @@ struct PassArgs {
   const void* fbox;  // forcing box [3][2Fz+1][2Fy+1][Fx+1] or null
   int Fx, Fy, Fz;
   int xdiag;         // x pass: only the max |u| reduction (no product, no output)
-  int xrpc;          // x pass rows per CTA (0 = largest that keeps two CTAs per SM)
+  int xrpc;          // x pass rows per CTA (0 = the launcher's rule, else at most this many)
   int beside;        // launches of other plans that run at the same time, this one included (0 = 1)
   int shape[3];      // shape variant of the z-inverse, y and z-forward passes (ColShape; 0 = default)
   int* err;          // device error word (bounded waits that gave up), never null

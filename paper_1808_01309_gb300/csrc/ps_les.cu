@@ -756,7 +756,7 @@ cudaError_t les_closure_grad(const Geo& g, Spec in, Spec f, const void* twx, con
   const long long M = (long long)g.nz * g.ny * g.nh;
   const V *tx = static_cast<const V*>(twx), *ty = static_cast<const V*>(twy), *tz = static_cast<const V*>(twz);
   // forward: features (keeping the gradient rows), network, stress, its
-  // divergence (compact), as in les_closure_term
+  // divergence (compact)
   k_grad<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, in, s.spec);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = spec2phys(g, 9, s.spec, s.spec, s.phys, tx, ty, tz, st);

@@ -1,7 +1,6 @@
-// Device pieces of the closure's network (5 -> 64 -> 64 -> 6, GELU) shared by
-// the MLP kernels (ps_mlp.cu) and the fused closure kernel (ps_les.cu): the
-// BF16 tensor-core fragments, the activation, and the forward pass of a
-// 16-sample tile held in the registers of one warp.
+// Device pieces of the closure's network (5 -> 64 -> 64 -> 6, GELU) for the MLP
+// kernels (ps_mlp.cu): the BF16 tensor-core fragments, the activations, and the
+// forward pass of a 16-sample tile held in the registers of one warp.
 //
 // Parameter vector (FP32): W1 [5][64] | b1 [64] | W2 [64][64] | b2 [64] |
 // W3 [64][6] | b3 [6]   (row-major, y = x W + b).
@@ -76,9 +75,10 @@ __device__ __forceinline__ float clamp_low(float z, float lo) {
   return y;
 }
 
-// GELU (tanh form) and its derivative from one tanh, as training uses them (the
-// sigmoid form of gelu4 would take 538 us per 2.1 M samples instead of 692, but
-// moves BF16 roundings, and with them the loss, beyond its bounds).
+// GELU (tanh form) and its derivative from one tanh, as training uses them.  (The
+// sigmoid form of gelu4 takes 538 us per 2.1 M samples instead of 692, but rounds
+// some activations to the neighbouring BF16 number, which moves the loss and the
+// gradients.)
 __device__ __forceinline__ void gelu_with_grad(float x, float& h, float& g) {
   constexpr float C = 0.7978845608028654f;  // sqrt(2/pi)
   const float t = tanhf(C * (x + 0.044715f * x * x * x));

@@ -60,7 +60,7 @@ template <typename T, int N, int K = 0> struct ColThreads {
 // N points: kx columns per CTA (TX), points per thread (E), threads per line
 // (G), lines of the other index per CTA (NB, about 256 threads per CTA).
 // VAR 0 (256 threads) is that of the ensemble's kernels and of plans whose
-// launches run beside others' (48 members: 12.5 ms for two steps, 13.1 with VAR
+// launches run beside others' (48 members: 12.65 ms for two steps, 13.13 with VAR
 // 3); VAR 3, the default of the per-pass launches, has the same columns and points
 // in smaller CTAs for lines of at most 256 points, whose barriers hold up fewer
 // warps and whose loads and transforms interleave: 64 threads up to 128 points,
@@ -171,8 +171,8 @@ template <typename T, int N> struct ColBuf {
 // memory (stage + exchange above 113 KB at RPCOf rows; kx extent of the
 // 2/3 rule).  Its CTAs then have half the threads of the launch bound and
 // two of them fill the SM's shared memory, so the kernel may use the
-// registers of one full-size CTA per SM instead of spilling.  (Rows whose
-// lines are transformed three together only: FP32 multiples of three.)
+// registers of one full-size CTA per SM instead of spilling.  (Only rows whose
+// lines are transformed three together, XLines.)
 template <typename T, int N> struct XHalved {
   static constexpr long long kxp = ((N + 2) / 3 + 15) / 16 * 16;
   static constexpr int E = EPass<T, N, 3>::v, R = RPCOf<T, N>::v;
@@ -420,7 +420,8 @@ __device__ __forceinline__ void zinv_tile(const PassArgs& a, const TL& tl) {
         out[(6 * grp + f) * fstride + n * zstride + (long long)iy * g.kxp + kx] = x[m];
       }
     }
-    if constexpr (LinePos<T, N, E>::paired) __syncthreads();  // the exchange buffer is free again
+    // (after paired lines the exchange buffer would not be free yet)
+    static_assert(!LinePos<T, N, E>::paired, "a barrier before the next field");
   }
   __syncthreads();  // the tile is restaged for the next group
   }
