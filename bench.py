@@ -930,13 +930,13 @@ def run_reference(args):
     value = nc ** 3 / t / 1e9
     desc = ("each step: " + cpu_sample_desc(nc, args.n, t, cpu_cores())
             + "; ms_per_step is the time of that sample, the work each timed step did")
-    line = {"impl": "reference", "metric": METRIC, "value": round(value, 6), "unit": UNIT, "n_gpus": args.gpus,
+    line = {"impl": "reference", "metric": METRIC, "value": round(value, 9), "unit": UNIT, "n_gpus": args.gpus,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(t * 1e3, 1),
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
             "data": "synthetic", "config": config_of(args.n, args.gpus),
-            "cpu_baseline": {"value": round(value, 6), "unit": UNIT, "cores": cpu_cores(), "kind": "oracle",
+            "cpu_baseline": {"value": round(value, 9), "unit": UNIT, "cores": cpu_cores(), "kind": "oracle",
                              "sample": desc},
-            "e2e": {"value": round(value, 6), "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
+            "e2e": {"value": round(value, 9), "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
     print(json.dumps(line), flush=True)
 
 
