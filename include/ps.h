@@ -87,8 +87,9 @@ typedef struct ps_plan ps_plan;
  *                transforms run in block fixed point: with S the sum of
  *                |re| + |im| over a line along an axis, each element is held to
  *                2^-61 S, which an FP64 transform's own rounding reaches at
- *                512 points, but to no less than 2^-1021: lines with S below
- *                2^-937 (1e-282) lose bits.  A line with an Inf or a NaN, or
+ *                512 points, but to no less than 2^-1021, as if subnormal
+ *                numbers were flushed to zero: lines with S below 2^-937
+ *                (1e-282) lose bits.  A line with an Inf or a NaN, or
  *                with S from 2^1024 on, becomes NaN as a whole; the sign of a
  *                zero is not kept
  *   eq         : PS_HD, or PS_MHD (Eqs. uMHD, bMHD: the state then has six
