@@ -648,8 +648,10 @@ ps_status ps_ensemble_tune(ps_ensemble* e, const void* const* uhats, double dt, 
       for (int k = 0; k < 3; ++k) plan_set_shape(p, k, 0);
     }
   };
-  default_shapes();
-  drop_graph(e);
+  if (st == PS_OK) {
+    default_shapes();
+    drop_graph(e);
+  }
   const auto time_graph = [&](double* ms) {
     return time_ms(e, 3, [&] { return run_graph(e, work.data(), dt, 0.0, 1); }, ms);
   };
