@@ -22,6 +22,8 @@
 
 namespace ps {
 void set_last_error(const std::string& msg);
+// The tables on the device are those of dt: a graph that computes them ran (ps_plan.cu).
+void plan_set_tables(ps_plan* p, double dt);
 }
 
 using namespace ps;
@@ -112,6 +114,21 @@ void drop_graph(ps_ensemble* e) {
   e->key_steps = -1;
 }
 
+// Launches a captured graph of all members' steps, which computes their factor
+// tables for its own dt at every replay.
+ps_status launch_graph(ps_ensemble* e, cudaGraphExec_t exec, double dt, double t_end) {
+  ENS_CU(cudaGraphLaunch(exec, e->main), "graph launch");
+  for (ps_plan* p : e->plans) {
+    plan_set_tables(p, dt);
+    plan_set_time(p, t_end);
+  }
+  return PS_OK;
+}
+// After a capture: what it recorded has not run.
+void forget_tables(ps_ensemble* e) {
+  for (ps_plan* p : e->plans) plan_invalidate_tables(p);
+}
+
 // Sequential: every member's steps on the ensemble stream, member by member.
 ps_status run_sequential(ps_ensemble* e, void* const* u, double dt, double t, int nsteps) {
   for (size_t i = 0; i < e->plans.size(); ++i) plan_set_stream(e->plans[i], e->main);
@@ -148,6 +165,7 @@ ps_status capture(ps_ensemble* e, void* const* u, double dt, double t, int nstep
   }
   cudaGraph_t g = nullptr;
   ce = cudaStreamEndCapture(e->cap, &g);
+  forget_tables(e);
   for (ps_plan* p : e->plans) plan_set_beside(p, 1);
   if (st != PS_OK) {
     if (g) cudaGraphDestroy(g);
@@ -173,9 +191,7 @@ ps_status run_graph(ps_ensemble* e, void* const* u, double dt, double t, int nst
     ps_status st = capture(e, u, dt, t, nsteps, e->nbranch);
     if (st != PS_OK) return st;
   }
-  ENS_CU(cudaGraphLaunch(e->exec, e->main), "graph launch");
-  for (ps_plan* p : e->plans) plan_set_time(p, t + nsteps * dt);
-  return PS_OK;
+  return launch_graph(e, e->exec, dt, t + nsteps * dt);
 }
 
 void drop_pgraph(ps_ensemble* e) {
@@ -350,6 +366,7 @@ ps_status persist_capture(ps_ensemble* e, void* const* u, double dt, int nsteps)
   }
   cudaGraph_t g = nullptr;
   ce = cudaStreamEndCapture(e->cap, &g);
+  forget_tables(e);
   if (st != PS_OK) {
     if (g) cudaGraphDestroy(g);
     return st;
@@ -370,9 +387,7 @@ ps_status run_persistent(ps_ensemble* e, void* const* u, double dt, double t, in
     ps_status st = persist_capture(e, u, dt, nsteps);
     if (st != PS_OK) return st;
   }
-  ENS_CU(cudaGraphLaunch(e->pexec, e->main), "graph launch");
-  for (ps_plan* p : e->plans) plan_set_time(p, t + nsteps * dt);
-  return PS_OK;
+  return launch_graph(e, e->pexec, dt, t + nsteps * dt);
 }
 
 void drop_bgraph(ps_ensemble* e) {
@@ -481,6 +496,7 @@ ps_status batch_capture(ps_ensemble* e, void* const* u, double dt, int nsteps) {
   }
   cudaGraph_t gr = nullptr;
   ce = cudaStreamEndCapture(e->cap, &gr);
+  forget_tables(e);
   if (st != PS_OK) {
     if (gr) cudaGraphDestroy(gr);
     return st;
@@ -501,9 +517,7 @@ ps_status run_batched(ps_ensemble* e, void* const* u, double dt, double t, int n
     ps_status st = batch_capture(e, u, dt, nsteps);
     if (st != PS_OK) return st;
   }
-  ENS_CU(cudaGraphLaunch(e->bexec, e->main), "graph launch");
-  for (ps_plan* p : e->plans) plan_set_time(p, t + nsteps * dt);
-  return PS_OK;
+  return launch_graph(e, e->bexec, dt, t + nsteps * dt);
 }
 
 // Average milliseconds of `reps` calls of f on the main stream.

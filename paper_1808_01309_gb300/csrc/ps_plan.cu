@@ -548,6 +548,7 @@ void plan_set_xrpc(ps_plan* p, int rpc) {
   p->xrpc = rpc;
 }
 void plan_invalidate_tables(ps_plan* p) { p->if_dt = NAN; }
+void plan_set_tables(ps_plan* p, double dt) { p->if_dt = dt; }
 bool plan_set_shape(ps_plan* p, int k, int var) {
   if (k < 0 || k > 2) return false;
   const int n = k == 1 ? p->g.ny : p->g.nz;
@@ -881,9 +882,9 @@ ps_status ps_rk_steps(ps_plan* p, void* uhat, double dt, double t, int nsteps) {
     cudaGraph_t g = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(p->cap, &g);
     p->stream = home;
+    p->if_dt = NAN;  // nothing has run yet
     if (st != PS_OK) {
       if (g) cudaGraphDestroy(g);
-      p->if_dt = NAN;
       return st;
     }
     PS_CU(ce, "end capture");
@@ -895,7 +896,9 @@ ps_status ps_rk_steps(ps_plan* p, void* uhat, double dt, double t, int nsteps) {
     p->g_launches = p->launches - l0;
     p->launches = l0;
   }
+  p->if_dt = NAN;
   PS_CU(cudaGraphLaunch(p->gexec, p->stream), "graph launch");
+  p->if_dt = dt;  // a replay computes the tables of its own dt
   p->launches += p->g_launches;
   p->time = t + nsteps * dt;
   return PS_OK;

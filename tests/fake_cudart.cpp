@@ -190,12 +190,13 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
   return cudaSuccess;
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
-  *e = reinterpret_cast<cudaGraphExec_t>(&token);
-  return cudaSuccess;
+  const cudaError_t r = result("cudaGraphInstantiate");
+  if (r == cudaSuccess) *e = reinterpret_cast<cudaGraphExec_t>(&token);
+  return r;
 }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) {
   ++graph_launches;
-  return cudaSuccess;
+  return result("cudaGraphLaunch");
 }
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }

@@ -247,3 +247,60 @@ def test_the_ensemble_tuner_times_the_kernels_that_the_graph_runs(fake, sizes):
         ps.ps_plan_destroy(plan)
     assert alone == set(_launches(fake, False))
     ps.ps_ensemble_destroy(e)
+
+
+def _tables(fake):
+    """Launches of the integrating-factor tables out of a capture."""
+    return sum("k_if_tables" in line and line.endswith(" 0") for line in fake.lib.fake_launches().decode().splitlines())
+
+
+def test_a_replayed_graph_leaves_the_tables_of_its_own_step(fake):
+    """A graph computes the factor tables of its dt at every replay: a single
+    step with another dt after it needs its own again."""
+    ps = fake.ps
+    plan, u = ps.ps_plan_create(ps.make_config(32, nu=1e-3)), np.zeros((3, 32, 32, 17), np.complex64).ctypes.data
+    ps.ps_rk_steps(plan, u, 1e-3, 0.0, 2)
+    ps.ps_rk_step(plan, u, 2e-3)
+    ps.ps_rk_steps(plan, u, 1e-3, 0.0, 2)  # replayed
+    fake.lib.fake_reset()
+    ps.ps_rk_step(plan, u, 2e-3)
+    assert _tables(fake) == 1
+    ps.ps_rk_step(plan, u, 2e-3)
+    assert _tables(fake) == 1
+    ps.ps_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("mode", ["ENS_GRAPH", "ENS_PERSISTENT", "ENS_BATCHED"])
+def test_a_replayed_ensemble_graph_leaves_the_tables_of_its_own_step(fake, mode):
+    calls = Calls(fake)
+    calls.prepare("persistent ensemble")
+    ps, e, states = fake.ps, calls.made[-1][1], [calls.u.ctypes.data] * 2
+
+    def step(dt, m):
+        ps.ps_ensemble_rk_steps(e, states, dt, 0.0, 1, getattr(ps, m))
+
+    for dt, m in ((1e-3, mode), (2e-3, "ENS_SEQUENTIAL"), (1e-3, mode)):
+        step(dt, m)
+    fake.lib.fake_reset()
+    step(2e-3, "ENS_SEQUENTIAL")
+    assert _tables(fake) == 2
+    calls.close()
+
+
+@pytest.mark.parametrize("call", ["cudaGraphInstantiate", "cudaGraphLaunch"])
+def test_tables_of_a_graph_that_did_not_run_are_not_taken_for_computed(fake, call):
+    ps = fake.ps
+    plan, u = ps.ps_plan_create(ps.make_config(32, nu=1e-3)), np.zeros((3, 32, 32, 17), np.complex64).ctypes.data
+    ens = ps.ps_ensemble_create([ps.make_config(32, nu=1e-3)])
+    fake.fail(call, 1, ILLEGAL_ADDRESS)
+    with pytest.raises(ps.PsError):
+        ps.ps_rk_steps(plan, u, 1e-3, 0.0, 2)
+    fake.fail(call, 1, ILLEGAL_ADDRESS)
+    with pytest.raises(ps.PsError):
+        ps.ps_ensemble_rk_steps(ens, [u], 1e-3, 0.0, 2, ps.ENS_GRAPH)
+    fake.lib.fake_reset()
+    ps.ps_rk_step(plan, u, 1e-3)
+    ps.ps_ensemble_rk_steps(ens, [u], 1e-3, 0.0, 1, ps.ENS_SEQUENTIAL)
+    assert _tables(fake) == 2
+    ps.ps_ensemble_destroy(ens)
+    ps.ps_plan_destroy(plan)
